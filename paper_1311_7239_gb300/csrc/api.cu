@@ -659,13 +659,17 @@ cudaError_t launch_step_at(const lbm_ctx* c, int cur, cudaStream_t s) {
   return c->inplace ? launch_step_inplace(P, c->prec, c->het, thermal_of(c), s) : launch_step(P, c->prec, c->het, thermal_of(c), s);
 }
 
+bool steps_in_pairs(const lbm_ctx* c) { return march_takes(params_for(c), c->prec, c->het, thermal_of(c)); }
+
 // Instantiate the graph of kGraphSteps steps that starts from buffer `cur`.
 int capture_graph(lbm_ctx* c, int cur) {
   if (!c->capture_stream) LBM_CUDA(cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking), "cudaStreamCreate");
   LBM_CUDA(cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
   cudaError_t launch_err = cudaSuccess;
-  for (int k = 0; k < kGraphSteps && launch_err == cudaSuccess; ++k)
-    launch_err = launch_step_at(c, cur ^ (k & 1), c->capture_stream);
+  const bool pairs = steps_in_pairs(c);
+  for (int k = 0; k < (pairs ? kGraphSteps / 2 : kGraphSteps) && launch_err == cudaSuccess; ++k)
+    launch_err = pairs ? launch_march(params_at(c, cur ^ (k & 1)), c->prec, c->het, thermal_of(c), c->capture_stream)
+                       : launch_step_at(c, cur ^ (k & 1), c->capture_stream);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(c->capture_stream, &g);
   if (launch_err != cudaSuccess || e != cudaSuccess) {
@@ -686,7 +690,8 @@ int capture_graph(lbm_ctx* c, int cur) {
 namespace {
 
 int run_steps(lbm_ctx* c, int n) {
-  while (n >= kGraphSteps) {  // replay a captured graph of kGraphSteps steps
+  const bool pairs = steps_in_pairs(c);
+  while (pairs ? n > kGraphSteps : n >= kGraphSteps) {  // replay a captured graph of kGraphSteps steps
     if (!c->graph[c->cur]) {
       int rc = capture_graph(c, c->cur);
       if (rc) return rc;
@@ -695,6 +700,12 @@ int run_steps(lbm_ctx* c, int n) {
     c->steps += kGraphSteps;
     c->history += kGraphSteps;
     n -= kGraphSteps;
+  }
+  for (; pairs && n > 2; n -= 2) {
+    LBM_CUDA(launch_march(params_at(c, c->cur), c->prec, c->het, thermal_of(c), c->stream), "step kernel");
+    c->cur ^= 1;
+    c->steps += 2;
+    c->history += 2;
   }
   for (int k = 0; k < n; ++k) {
     LBM_CUDA(launch_step_at(c, c->cur, c->stream), "step kernel");

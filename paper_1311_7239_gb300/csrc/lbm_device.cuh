@@ -447,6 +447,86 @@ __device__ __forceinline__ void collide_pair(float2 d[8], const PairCoef& c, flo
   d[7] = add2(d[7], add2(H, PM));
 }
 
+// collide_d2q8 for two cells at once on the packed FP32 pairs, in true units and with the roundings
+// of the scalar form operation by operation (the multiply-adds it is compiled to, written out), so
+// that both give the same bits: FP32 storage may take either.  Differences are multiply-adds by -1,
+// since the packed instructions have no negated operands.
+struct PairMedium {
+  float2 phi, inv_phi, l0, l1, nclin, ncnl, s_v;  // l0 = 1/2 + c_lin / 4, l1 = c_nl / 2, -c_lin, -c_nl
+};
+__device__ __forceinline__ float2 less2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.0f), a); }  // a - b
+
+__device__ __forceinline__ PairMedium pair_medium(const Coef& a, const Coef& b) {
+  PairMedium m;
+  m.phi = make_float2(a.phi, b.phi);
+  m.inv_phi = make_float2(a.inv_phi, b.inv_phi);
+  m.l0 = make_float2(__fmaf_rn(0.25f, a.c_lin, 0.5f), __fmaf_rn(0.25f, b.c_lin, 0.5f));
+  m.l1 = make_float2(0.5f * a.c_nl, 0.5f * b.c_nl);
+  m.nclin = make_float2(-a.c_lin, -b.c_lin);
+  m.ncnl = make_float2(-a.c_nl, -b.c_nl);
+  m.s_v = make_float2(a.s_v, b.s_v);
+  return m;
+}
+
+__device__ __forceinline__ void collide_d2q8_pair(float2 d[8], const PairMedium& c, float ax, float2 ay, const StepParams& P, float2& ux,
+                                                  float2& uy) {
+  const float rho0 = P.rho0;
+  // m = M d, Eq. 10 (n13, n24: -(d1 - d3), -(d2 - d4))
+  const float2 a13 = add2(d[0], d[2]), a24 = add2(d[1], d[3]);
+  const float2 n13 = less2(d[2], d[0]), n24 = less2(d[3], d[1]);
+  const float2 s57 = add2(d[4], d[6]), s68 = add2(d[5], d[7]);
+  const float2 t57 = less2(d[4], d[6]), t68 = less2(d[5], d[7]);
+  const float2 diag = add2(s57, s68), A = add2(a13, a24);
+  const float2 m1 = add2(A, diag), m2 = less2(diag, A);
+  const float2 dxs = less2(t57, t68), dys = add2(t57, t68);
+  const float2 m3 = less2(dxs, n13), m5 = less2(dys, n24);
+  const float2 m7 = less2(a13, a24), m8 = less2(s57, s68);
+  // Eqs. 17-19
+  const float2 h = mul2(f2(0.5f), c.phi);
+  const float2 vx = fma2(h, f2(ax), mul2(m3, f2(P.inv_rho0))), vy = fma2(h, ay, mul2(m5, f2(P.inv_rho0)));
+  const float2 vsq = fma2(vx, vx, mul2(vy, vy));
+  const float2 vmag = make_float2(fast_sqrt(vsq.x), fast_sqrt(vsq.y));
+  const float2 R = fma2(c.l0, c.l0, mul2(c.l1, vmag));  // >= l0^2 >= 1/4
+  // (scalar products: a packed product would be fused with the sum)
+  const float2 den = add2(c.l0, make_float2(__fmul_rn(R.x, rsqrtf(R.x)), __fmul_rn(R.y, rsqrtf(R.y))));
+  const float2 inv = make_float2(fast_rcp(den.x), fast_rcp(den.y));
+  ux = mul2(vx, inv);
+  uy = mul2(vy, inv);
+  const float2 umag = mul2(vmag, inv), nuy = mul2(uy, f2(-1.0f));
+  // Eq. 20 (phi p = 0.6 Y) and Eq. 3
+  const float2 usq = fma2(ux, ux, mul2(uy, uy));
+  const float2 Y = fma2(mul2(f2(-(2.0f / 3.0f) * rho0), usq), c.inv_phi, m1);
+  const float2 nd = fma2(c.ncnl, umag, c.nclin);
+  const float2 Fx = fma2(c.phi, f2(ax), mul2(nd, ux)), Fy = fma2(c.phi, ay, mul2(nd, uy));
+  // Eqs. 11-14 as increments (collide_d2q8)
+  const float2 rFx = mul2(f2(rho0), Fx), rFy = mul2(f2(rho0), Fy);
+  const float be = __fmaf_rn(-0.5f, P.s_e, 1.0f), nbq = -__fmaf_rn(-0.5f, P.s_q, 1.0f);
+  const float2 S2 = mul2(mul2(f2(rho0 * 0.8f), fma2(ux, Fx, mul2(uy, Fy))), c.inv_phi);
+  const float2 k2 = fma2(f2(be), S2, mul2(f2(-P.s_e), fma2(f2(0.6f), Y, m2)));
+  const float2 gx = fma2(f2(0.5f), rFx, fma2(f2(2.0f), dxs, n13)), gy = fma2(f2(0.5f), rFy, fma2(f2(2.0f), dys, n24));
+  const float2 k4 = fma2(f2(-P.s_q), gx, mul2(f2(nbq), rFx)), k6 = fma2(f2(-P.s_q), gy, mul2(f2(nbq), rFy));
+  const float2 hv = fma2(f2(-0.5f), c.s_v, f2(1.0f)), nsv = mul2(f2(-1.0f), c.s_v);
+  const float2 A7 = fma2(mul2(f2(-rho0), fma2(ux, ux, mul2(nuy, uy))), c.inv_phi, m7);
+  const float2 Z7 = mul2(mul2(mul2(hv, f2(2.0f)), f2(rho0)), fma2(ux, Fx, mul2(nuy, Fy)));
+  const float2 k7 = fma2(Z7, c.inv_phi, mul2(nsv, A7));
+  const float2 A8 = fma2(mul2(mul2(f2(-rho0), ux), uy), c.inv_phi, m8);
+  const float2 Z8 = mul2(mul2(hv, f2(rho0)), fma2(ux, Fy, mul2(uy, Fx)));
+  const float2 k8 = fma2(Z8, c.inv_phi, mul2(nsv, A8));
+  // d+ = d + M^-1 k
+  const float2 q2 = mul2(k2, f2(0.125f)), q7 = mul2(k7, f2(0.25f)), q8 = mul2(k8, f2(0.25f));
+  const float2 q4 = mul2(k4, f2(1.0f / 12.0f)), q6 = mul2(k6, f2(1.0f / 12.0f));
+  const float2 X = fma2(rFx, f2(1.0f / 6.0f), mul2(f2(-2.0f), q4)), Yy = fma2(rFy, f2(1.0f / 6.0f), mul2(f2(-2.0f), q6));
+  const float2 Px = fma2(rFx, f2(1.0f / 6.0f), q4), Py = fma2(rFy, f2(1.0f / 6.0f), q6);
+  d[0] = add2(d[0], less2(add2(X, q7), q2));
+  d[1] = add2(d[1], less2(less2(Yy, q7), q2));
+  d[2] = add2(d[2], less2(less2(q7, X), q2));
+  d[3] = less2(d[3], add2(add2(Yy, q7), q2));
+  d[4] = add2(d[4], add2(add2(add2(Px, Py), q8), q2));
+  d[5] = add2(d[5], add2(less2(less2(Py, Px), q8), q2));
+  d[6] = add2(d[6], add2(less2(less2(q8, Px), Py), q2));
+  d[7] = add2(d[7], add2(less2(less2(Px, Py), q8), q2));
+}
+
 // macroscopic quantities only (no collision), for read-out kernels
 __device__ __forceinline__ Macro macro_d2q8(const float d[8], const Coef& c, float ax, float ay, float rho0) {
   Macro r;
@@ -518,6 +598,22 @@ __device__ __forceinline__ void collide_d2q5_pair(float2 g[5], float2 ux, float2
   g[2] = add2(g[2], add2(r2, b));
   g[3] = add2(g[3], sub2(a, r1));
   g[4] = add2(g[4], sub2(b, r2));
+}
+
+// collide_d2q5 for two cells at once, rounded as the scalar form (see collide_d2q8_pair); n0 = T - T0.
+__device__ __forceinline__ void collide_d2q5_pair_fp32(float2 g[5], float2 n0, float2 ux, float2 uy, const StepParams& P) {
+  const float2 n1 = less2(g[1], g[3]), n2 = less2(g[2], g[4]);
+  const float2 n3 = fma2(f2(-4.0f), g[0], add2(add2(add2(g[1], g[2]), g[3]), g[4]));
+  const float2 n4 = less2(add2(less2(g[1], g[2]), g[3]), g[4]);
+  const float2 T = add2(f2(P.T0), n0), nT = mul2(T, f2(-1.0f));
+  const float2 b1 = fma2(mul2(ux, nT), f2(P.inv_sigma), n1), b2 = fma2(mul2(uy, nT), f2(P.inv_sigma), n2);
+  const float2 r3 = mul2(f2(-0.05f * P.zeta3), fma2(f2(-P.varpi), T, n3));
+  const float2 z1 = f2(-0.5f * P.zeta1), nz1 = f2(0.5f * P.zeta1), z4 = f2(-0.25f * P.zeta4), nz4 = f2(0.25f * P.zeta4);
+  g[0] = fma2(f2(-4.0f), r3, g[0]);
+  g[1] = add2(g[1], fma2(z4, n4, fma2(z1, b1, r3)));
+  g[2] = add2(g[2], fma2(nz4, n4, fma2(z1, b2, r3)));
+  g[3] = add2(g[3], fma2(z4, n4, fma2(nz1, b1, r3)));
+  g[4] = add2(g[4], fma2(nz4, n4, fma2(nz1, b2, r3)));
 }
 
 // D2Q5 velocities of Eq. B.3 (0 rest, 1..4 as D2Q8's first four)
@@ -619,6 +715,28 @@ __device__ __forceinline__ float wall_term(const StepParams& P, int i, int w) {
   return 6.0f * w_of(i) * P.rho0 * ((float)ex_of(i) * __ldg(P.uw + 2 * w) + (float)ey_of(i) * __ldg(P.uw + 2 * w + 1));
 }
 
+// e_i . u_w of wall w
+__device__ __forceinline__ float wall_dot(const StepParams& P, int i, int w) {
+  return __fadd_rn((float)ex_of(i) * __ldg(P.uw + 2 * w), (float)ey_of(i) * __ldg(P.uw + 2 * w + 1));
+}
+
+// Halfway bounce-back: f_i(x) = f+_opp(i)(x) + 2 w_i rho0 (e_i . u_w) / c_s^2 with own = f+_opp(i)(x),
+// dot = e_i . u_w; and its counterpart for the temperature, anti-bounce-back at a wall with a prescribed
+// temperature (deviation form of g_i = -g+_opp + 2 T_w / 5, reference T0 / 5), bounce-back at an adiabatic
+// one.  The roundings are written out so that every kernel that applies a wall gives the same bits (with
+// FP16 storage the scale's product is part of own, and the wall term is rounded before it is added).
+template <int PREC>
+__device__ __forceinline__ float bounce(const StepParams& P, float own, int i, float dot) {
+  const float c = 6.0f * w_of(i) * P.rho0;
+  return PREC == PREC_FP16 ? __fadd_rn(own, __fmul_rn(c, dot)) : __fmaf_rn(c, dot, own);
+}
+template <int PREC>
+__device__ __forceinline__ float heat_bounce(const StepParams& P, float own, int w) {
+  if (!P.Tdir[w]) return own;
+  const float d = P.Tw[w] - P.T0;
+  return PREC == PREC_FP16 ? __fadd_rn(-own, __fmul_rn(0.4f, d)) : __fmaf_rn(0.4f, d, -own);
+}
+
 template <int PREC>
 __device__ __forceinline__ float pull_one(const StepParams& P, const typename Store<PREC>::T* src, int x, int y, int i) {
   using S = Store<PREC>;
@@ -633,11 +751,8 @@ __device__ __forceinline__ float pull_one(const StepParams& P, const typename St
   if (P.bc_y != BC_WALL) sy = (sy + P.ny) % P.ny;
   if (sx >= 0 && sx < P.nx && sy >= 0 && sy < P.ny)
     return S::dec(src[(int64_t)i * P.plane + (int64_t)sy * P.pitch + sx], P.inv_scale);
-  // halfway bounce-back: f_i(x) = f+_opp(i)(x) + 2 w_i rho0 (e_i . u_w) / c_s^2
   const int w = wall_of(sx, sy, P.ny);
-  const int o = opp_of(i);
-  const float own = S::dec(src[(int64_t)o * P.plane + (int64_t)y * P.pitch + x], P.inv_scale);
-  return own + 6.0f * w_of(i) * P.rho0 * ((float)ex_of(i) * __ldg(P.uw + 2 * w) + (float)ey_of(i) * __ldg(P.uw + 2 * w + 1));
+  return bounce<PREC>(P, S::dec(src[(int64_t)opp_of(i) * P.plane + (int64_t)y * P.pitch + x], P.inv_scale), i, wall_dot(P, i, w));
 }
 
 template <int PREC>
@@ -663,9 +778,7 @@ __device__ __forceinline__ float pull_one_g(const StepParams& P, const typename 
   if (sx >= 0 && sx < P.nx && sy >= 0 && sy < P.ny)
     return S::dec(src[(int64_t)i * P.plane + (int64_t)sy * P.pitch + sx], P.inv_scale);
   const int w = wall_of(sx, sy, P.ny);
-  const float own = S::dec(src[(int64_t)opp5(i) * P.plane + (int64_t)y * P.pitch + x], P.inv_scale);
-  // deviation form of g_i = -g+_opp + 2 T_w / 5 (reference T0 / 5): d_i = -d+_opp + 2 (T_w - T0) / 5
-  return P.Tdir[w] ? (-own + 0.4f * (P.Tw[w] - P.T0)) : own;
+  return heat_bounce<PREC>(P, S::dec(src[(int64_t)opp5(i) * P.plane + (int64_t)y * P.pitch + x], P.inv_scale), w);
 }
 
 template <int PREC>

@@ -37,6 +37,8 @@ int batch_max_ctas_per_sm(int prec, int nt);
 cudaError_t launch_step_batch(const StepParams* Pd, const int64_t* item_start, const int* item_lattice, int n, int64_t total, int prec,
                               int nt, int grid, int flat, cudaStream_t s);
 cudaError_t launch_step(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);
+bool march_takes(const StepParams& P, int prec, bool het, bool thermal);
+cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);
 cudaError_t launch_step_inplace(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);
 int64_t inplace_items(int nx, int ny, int bc_x, int bc_y);
 cudaError_t launch_step_batch_inplace(const StepParams* Pd, const int64_t* item_start, const int* item_lattice, int64_t total, int prec,
