@@ -166,7 +166,9 @@ struct lbm_ctx {
 
 namespace {
 
-constexpr int kGraphSteps = 32;  // steps per captured graph (even: a replay ends on the buffer it began on)
+// Steps per captured graph (a replay ends on the buffer it began on).  A replay costs 2.6 us beside its
+// kernels, which a small lattice notices.
+constexpr int kGraphSteps = 32, kTileGraphSteps = 128;
 
 bool thermal_of(const lbm_ctx* c) { return c->cfg.thermal != 0; }
 
@@ -659,17 +661,36 @@ cudaError_t launch_step_at(const lbm_ctx* c, int cur, cudaStream_t s) {
   return c->inplace ? launch_step_inplace(P, c->prec, c->het, thermal_of(c), s) : launch_step(P, c->prec, c->het, thermal_of(c), s);
 }
 
-bool steps_in_pairs(const lbm_ctx* c) { return march_takes(params_for(c), c->prec, c->het, thermal_of(c)); }
+// Steps that one launch takes for this context: up to `most`, several in shared memory (tile: small
+// lattices) or two (large ones), or one.
+struct Pace {
+  int most;
+  bool tile;
+  int graph;  // steps per captured graph
+};
 
-// Instantiate the graph of kGraphSteps steps that starts from buffer `cur`.
+Pace pace_of(const lbm_ctx* c) {
+  const StepParams P = params_for(c);
+  const int tile = tile_steps(P, c->prec, c->het, thermal_of(c));
+  if (tile > 1) return {tile, true, kTileGraphSteps};
+  return {march_takes(P, c->prec, c->het, thermal_of(c)) ? 2 : 1, false, kGraphSteps};
+}
+
+// `steps` steps, at most pace.most, from buffer `cur` into the other one
+cudaError_t launch_steps_at(const lbm_ctx* c, int cur, int steps, const Pace& pace, cudaStream_t s) {
+  if (steps == 1) return launch_step_at(c, cur, s);
+  const StepParams P = params_at(c, cur);
+  return pace.tile ? launch_tile(P, c->prec, c->het, thermal_of(c), steps, s) : launch_march(P, c->prec, c->het, thermal_of(c), s);
+}
+
+// Instantiate the graph of pace.graph steps that starts from buffer `cur`.
 int capture_graph(lbm_ctx* c, int cur) {
   if (!c->capture_stream) LBM_CUDA(cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking), "cudaStreamCreate");
   LBM_CUDA(cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
   cudaError_t launch_err = cudaSuccess;
-  const bool pairs = steps_in_pairs(c);
-  for (int k = 0; k < (pairs ? kGraphSteps / 2 : kGraphSteps) && launch_err == cudaSuccess; ++k)
-    launch_err = pairs ? launch_march(params_at(c, cur ^ (k & 1)), c->prec, c->het, thermal_of(c), c->capture_stream)
-                       : launch_step_at(c, cur ^ (k & 1), c->capture_stream);
+  const Pace pace = pace_of(c);
+  for (int k = 0; k < pace.graph / pace.most && launch_err == cudaSuccess; ++k)
+    launch_err = launch_steps_at(c, cur ^ (k & 1), pace.most, pace, c->capture_stream);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(c->capture_stream, &g);
   if (launch_err != cudaSuccess || e != cudaSuccess) {
@@ -690,28 +711,28 @@ int capture_graph(lbm_ctx* c, int cur) {
 namespace {
 
 int run_steps(lbm_ctx* c, int n) {
-  const bool pairs = steps_in_pairs(c);
-  while (pairs ? n > kGraphSteps : n >= kGraphSteps) {  // replay a captured graph of kGraphSteps steps
+  // Launches of several steps leave the state before the last of them nowhere, and the residual needs
+  // the state before the last step: that one is always taken by itself.
+  const Pace pace = pace_of(c);
+  const int most = pace.most;
+  while (most > 1 ? n > pace.graph : n >= pace.graph) {  // replay a captured graph
     if (!c->graph[c->cur]) {
       int rc = capture_graph(c, c->cur);
       if (rc) return rc;
     }
     LBM_CUDA(cudaGraphLaunch(c->graph[c->cur], c->stream), "cudaGraphLaunch");
-    c->steps += kGraphSteps;
-    c->history += kGraphSteps;
-    n -= kGraphSteps;
+    c->steps += pace.graph;
+    c->history += pace.graph;
+    n -= pace.graph;
   }
-  for (; pairs && n > 2; n -= 2) {
-    LBM_CUDA(launch_march(params_at(c, c->cur), c->prec, c->het, thermal_of(c), c->stream), "step kernel");
+  while (n > 0) {
+    int k = n - 1 < most ? n - 1 : most;
+    if (k < 1) k = 1;
+    LBM_CUDA(launch_steps_at(c, c->cur, k, pace, c->stream), "step kernel");
     c->cur ^= 1;
-    c->steps += 2;
-    c->history += 2;
-  }
-  for (int k = 0; k < n; ++k) {
-    LBM_CUDA(launch_step_at(c, c->cur, c->stream), "step kernel");
-    c->cur ^= 1;
-    ++c->steps;
-    ++c->history;
+    c->steps += k;
+    c->history += k;
+    n -= k;
   }
   return LBM_OK;
 }

@@ -215,6 +215,19 @@ struct Coef {
 __device__ __forceinline__ float fast_rcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ float fast_sqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
 
+// The same for arguments known to be normal numbers (or inf, NaN): without the instructions that scale
+// subnormal ones.
+__device__ __forceinline__ float rcp_normal(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 __device__ __forceinline__ float f4_get(const float4& v, int c) { return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w; }
 
 // Coefficients of a cell with porosity ph, permeability k and viscous rate sv (Eqs. 3-4, 13).
@@ -287,15 +300,24 @@ __device__ __forceinline__ void collide_d2q8(float d[8], const Coef& c, float ax
   const float m7 = a13 - a24;               // p_xx
   const float m8 = s57 - s68;               // p_xy
 
-  float ux, uy, umag;
-  velocity_from_j(m3, m5, c, ax, ay, P.inv_rho0, ux, uy, umag);
-  const float usq = ux * ux + uy * uy;
-  // Eq. 20 with c_s^2 / (1 - w0) = 3/5 and s0 = -2|u|^2 / (3 phi): phi p = 3/5 (sum f - 2/3 rho0 |u|^2 / phi)
-  const float phip_dev = 0.6f * (m1 - (2.0f / 3.0f) * rho0 * usq * c.inv_phi);
+  // (from here the multiply-adds are written out: the collision of two cells at once, and every kernel,
+  // must round as this one does)
+  const float h = 0.5f * c.phi;
+  const float vx = __fmaf_rn(h, ax, __fmul_rn(m3, P.inv_rho0)), vy = __fmaf_rn(h, ay, __fmul_rn(m5, P.inv_rho0));
+  const float l0 = __fmaf_rn(0.25f, c.c_lin, 0.5f), l1 = 0.5f * c.c_nl;
+  const float vmag = fast_sqrt(__fmaf_rn(vx, vx, __fmul_rn(vy, vy)));
+  // Eq. 18, the cancellation-free root of l1 |u|^2 + 2 l0 |u| - |v| = 0
+  const float R = __fmaf_rn(l0, l0, __fmul_rn(l1, vmag));  // >= l0^2 >= 1/4
+  const float inv = rcp_normal(__fadd_rn(l0, __fmul_rn(R, rsqrt_normal(R))));
+  const float ux = vx * inv, uy = vy * inv, umag = vmag * inv;
+  const float uy2 = uy * uy, usq = __fmaf_rn(ux, ux, uy2);
+  // Eq. 20 with c_s^2 / (1 - w0) = 3/5 and s0 = -2|u|^2 / (3 phi): phi p = 3/5 Y, Y = sum f - 2/3 rho0 |u|^2 / phi
+  const float Y = __fmaf_rn(-__fmul_rn((2.0f / 3.0f) * rho0, usq), c.inv_phi, m1);
+  const float phip_dev = 0.6f * Y;
   // Eq. 3
-  const float drag = c.c_lin + c.c_nl * umag;
-  const float Fx = -drag * ux + c.phi * ax;
-  const float Fy = -drag * uy + c.phi * ay;
+  const float drag = __fmaf_rn(c.c_nl, umag, c.c_lin);
+  const float Fx = __fmaf_rn(c.phi, ax, __fmul_rn(-drag, ux));
+  const float Fy = __fmaf_rn(c.phi, ay, __fmul_rn(-drag, uy));
 
   // Eqs. 11-14 as increments k = m+ - m = -Lambda (m - m_eq) + (I - Lambda/2) S.  m1 is conserved
   // (m1_eq = m1, S1 = 0); m3, m5 gain rho0 F for any s3, s5.  The q moments relax towards
@@ -304,27 +326,28 @@ __device__ __forceinline__ void collide_d2q8(float d[8], const Coef& c, float ax
   // them from m+) keeps FP32 rounding at about one unit of d per step.
   const float s_e = P.s_e, s_q = P.s_q, s_v = c.s_v;
   const float rFx = rho0 * Fx, rFy = rho0 * Fy;
-  const float S2 = rho0 * 0.8f * (ux * Fx + uy * Fy) * c.inv_phi;
-  const float k2 = -s_e * (m2 + phip_dev) + (1.0f - 0.5f * s_e) * S2;  // e_eq = -phi p
-  const float k3 = rFx;
-  const float k4 = -s_q * ((2.0f * dxs - d13) + 0.5f * rFx) - (1.0f - 0.5f * s_q) * rFx;
-  const float k5 = rFy;
-  const float k6 = -s_q * ((2.0f * dys - d24) + 0.5f * rFy) - (1.0f - 0.5f * s_q) * rFy;
-  const float hv = 1.0f - 0.5f * s_v;
-  const float k7 = -s_v * (m7 - rho0 * (ux * ux - uy * uy) * c.inv_phi) + hv * 2.0f * rho0 * (ux * Fx - uy * Fy) * c.inv_phi;
-  const float k8 = -s_v * (m8 - rho0 * ux * uy * c.inv_phi) + hv * rho0 * (ux * Fy + uy * Fx) * c.inv_phi;
+  const float be = __fmaf_rn(-0.5f, s_e, 1.0f), bq = __fmaf_rn(-0.5f, s_q, 1.0f), hv = __fmaf_rn(-0.5f, s_v, 1.0f);
+  const float S2 = __fmul_rn(__fmul_rn(rho0 * 0.8f, __fmaf_rn(ux, Fx, __fmul_rn(uy, Fy))), c.inv_phi);
+  const float k2 = __fmaf_rn(be, S2, __fmul_rn(-s_e, __fmaf_rn(0.6f, Y, m2)));  // e_eq = -phi p
+  const float gx = __fmaf_rn(0.5f, rFx, __fmaf_rn(2.0f, dxs, -d13)), gy = __fmaf_rn(0.5f, rFy, __fmaf_rn(2.0f, dys, -d24));
+  const float k4 = __fmaf_rn(-s_q, gx, -__fmul_rn(bq, rFx)), k6 = __fmaf_rn(-s_q, gy, -__fmul_rn(bq, rFy));
+  const float A7 = __fmaf_rn(-__fmul_rn(rho0, __fmaf_rn(ux, ux, -uy2)), c.inv_phi, m7);
+  const float Z7 = __fmul_rn(__fmul_rn(hv * 2.0f, rho0), __fmaf_rn(ux, Fx, -__fmul_rn(uy, Fy)));
+  const float k7 = __fmaf_rn(Z7, c.inv_phi, -__fmul_rn(s_v, A7));
+  const float A8 = __fmaf_rn(-__fmul_rn(__fmul_rn(rho0, ux), uy), c.inv_phi, m8);
+  const float Z8 = __fmul_rn(__fmul_rn(hv, rho0), __fmaf_rn(ux, Fy, __fmul_rn(uy, Fx)));
+  const float k8 = __fmaf_rn(Z8, c.inv_phi, -__fmul_rn(s_v, A8));
 
-  // d+ = d + M^-1 k, M^-1 = M^T diag(1/8, 1/8, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4), k1 = 0
+  // d+ = d + M^-1 k, M^-1 = M^T diag(1/8, 1/8, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4), k1 = 0, k3 = rFx, k5 = rFy
   const float q2 = k2 * 0.125f;
-  const float q3 = k3 * (1.0f / 6.0f), q4 = k4 * (1.0f / 12.0f);
-  const float q5 = k5 * (1.0f / 6.0f), q6 = k6 * (1.0f / 12.0f);
+  const float q4 = __fmul_rn(k4, 1.0f / 12.0f), q6 = __fmul_rn(k6, 1.0f / 12.0f);
   const float q7 = k7 * 0.25f, q8 = k8 * 0.25f;
-  const float X = q3 - 2.0f * q4, Y = q5 - 2.0f * q6;
-  const float Px = q3 + q4, Py = q5 + q6;
+  const float X = __fmaf_rn(rFx, 1.0f / 6.0f, -2.0f * q4), Y3 = __fmaf_rn(rFy, 1.0f / 6.0f, -2.0f * q6);
+  const float Px = __fmaf_rn(rFx, 1.0f / 6.0f, q4), Py = __fmaf_rn(rFy, 1.0f / 6.0f, q6);
   d[0] += (X + q7) - q2;
-  d[1] += (Y - q7) - q2;
+  d[1] += (Y3 - q7) - q2;
   d[2] += (q7 - X) - q2;
-  d[3] += (-Y - q7) - q2;
+  d[3] += (-Y3 - q7) - q2;
   d[4] += (Px + Py + q8) + q2;
   d[5] += (Py - Px - q8) + q2;
   d[6] += (q8 - Px - Py) + q2;
@@ -412,8 +435,8 @@ __device__ __forceinline__ void collide_pair(float2 d[8], const PairCoef& c, flo
   const float2 vsq = fma2(vx, vx, mul2(vy, vy));
   const float2 vmag = mul2(vsq, make_float2(vsq.x > 0.0f ? rsqrtf(vsq.x) : 0.0f, vsq.y > 0.0f ? rsqrtf(vsq.y) : 0.0f));
   const float2 t = fma2(c.l1, vmag, c.l0sq);  // >= l0^2 >= 1/4
-  const float2 den = add2(c.l0, mul2(t, make_float2(rsqrtf(t.x), rsqrtf(t.y))));
-  const float2 inv = make_float2(fast_rcp(den.x), fast_rcp(den.y));
+  const float2 den = add2(c.l0, mul2(t, make_float2(rsqrt_normal(t.x), rsqrt_normal(t.y))));
+  const float2 inv = make_float2(rcp_normal(den.x), rcp_normal(den.y));
   ux = mul2(vx, inv);
   uy = mul2(vy, inv);
   const float2 umag = mul2(vmag, inv);
@@ -488,8 +511,8 @@ __device__ __forceinline__ void collide_d2q8_pair(float2 d[8], const PairMedium&
   const float2 vmag = make_float2(fast_sqrt(vsq.x), fast_sqrt(vsq.y));
   const float2 R = fma2(c.l0, c.l0, mul2(c.l1, vmag));  // >= l0^2 >= 1/4
   // (scalar products: a packed product would be fused with the sum)
-  const float2 den = add2(c.l0, make_float2(__fmul_rn(R.x, rsqrtf(R.x)), __fmul_rn(R.y, rsqrtf(R.y))));
-  const float2 inv = make_float2(fast_rcp(den.x), fast_rcp(den.y));
+  const float2 den = add2(c.l0, make_float2(__fmul_rn(R.x, rsqrt_normal(R.x)), __fmul_rn(R.y, rsqrt_normal(R.y))));
+  const float2 inv = make_float2(rcp_normal(den.x), rcp_normal(den.y));
   ux = mul2(vx, inv);
   uy = mul2(vy, inv);
   const float2 umag = mul2(vmag, inv), nuy = mul2(uy, f2(-1.0f));
@@ -564,16 +587,15 @@ __device__ __forceinline__ float collide_d2q5(float g[5], float ux, float uy, co
   const float n4 = g[1] - g[2] + g[3] - g[4];
   const float T = P.T0 + n0;
   // increments n+ - n (n0 conserved), then g+ = g + N^-1 (n+ - n) with
-  // N^-1 = N^T diag(1/5, 1/2, 1/2, 1/20, 1/4)
-  const float r1 = -0.5f * P.zeta1 * (n1 - ux * T * P.inv_sigma);
-  const float r2 = -0.5f * P.zeta1 * (n2 - uy * T * P.inv_sigma);
-  const float r3 = -0.05f * P.zeta3 * (n3 - P.varpi * T);
-  const float r4 = -0.25f * P.zeta4 * n4;
-  g[0] += -4.0f * r3;
-  g[1] += (r1 + r3) + r4;
-  g[2] += (r2 + r3) - r4;
-  g[3] += (r3 - r1) + r4;
-  g[4] += (r3 - r2) - r4;
+  // N^-1 = N^T diag(1/5, 1/2, 1/2, 1/20, 1/4); multiply-adds written out (see collide_d2q8)
+  const float z1 = -0.5f * P.zeta1, z4 = -0.25f * P.zeta4;
+  const float b1 = __fmaf_rn(-__fmul_rn(ux, T), P.inv_sigma, n1), b2 = __fmaf_rn(-__fmul_rn(uy, T), P.inv_sigma, n2);
+  const float r3 = __fmul_rn(-0.05f * P.zeta3, __fmaf_rn(-P.varpi, T, n3));
+  g[0] = __fmaf_rn(-4.0f, r3, g[0]);
+  g[1] += __fmaf_rn(z4, n4, __fmaf_rn(z1, b1, r3));
+  g[2] += __fmaf_rn(-z4, n4, __fmaf_rn(z1, b2, r3));
+  g[3] += __fmaf_rn(z4, n4, __fmaf_rn(-z1, b1, r3));
+  g[4] += __fmaf_rn(-z4, n4, __fmaf_rn(-z1, b2, r3));
   return T;
 }
 

@@ -37,7 +37,10 @@ int batch_max_ctas_per_sm(int prec, int nt);
 cudaError_t launch_step_batch(const StepParams* Pd, const int64_t* item_start, const int* item_lattice, int n, int64_t total, int prec,
                               int nt, int grid, int flat, cudaStream_t s);
 cudaError_t launch_step(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);
+int sm_count();  // SMs of the current device
 bool march_takes(const StepParams& P, int prec, bool het, bool thermal);
+int tile_steps(const StepParams& P, int prec, bool het, bool thermal);
+cudaError_t launch_tile(const StepParams& P, int prec, bool het, bool thermal, int steps, cudaStream_t s);
 cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);
 cudaError_t launch_step_inplace(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);
 int64_t inplace_items(int nx, int ny, int bc_x, int bc_y);

@@ -14,114 +14,10 @@
 // pass was bound by instruction issue (79 %, 195 thread instructions per cell and step).
 // Measured (GLUPS, one step per pass -> two): FP32 4096^2 104 -> 178, per-cell medium 90 -> 147,
 // temperature (2048^2) 59 -> 95.  Every cell is rounded as by k_step: the results are the same bits.
-#include "lbm_device.cuh"
 #include "lbm_internal.h"
-#include "tiles.cuh"
+#include "rows.cuh"
 
 namespace lbm {
-
-// C consecutive cells of one population as stored: floats, or 32-bit words of two 16-bit values.
-template <int PREC, int C>
-struct Cells {
-  static_assert(C == 2 || C == 4, "cells per lane");
-  static constexpr int N = PREC == PREC_FP32 ? C : C / 2;
-  uint32_t v[N];
-};
-
-template <int PREC, int C>
-__device__ __forceinline__ Cells<PREC, C> load_cells(const typename Store<PREC>::T* __restrict__ p) {
-  Cells<PREC, C> r;
-  if constexpr (Cells<PREC, C>::N == 4) {
-    const uint4 q = *reinterpret_cast<const uint4*>(p);
-    r.v[0] = q.x; r.v[1] = q.y; r.v[2] = q.z; r.v[3] = q.w;
-  } else if constexpr (Cells<PREC, C>::N == 2) {
-    const uint2 q = *reinterpret_cast<const uint2*>(p);
-    r.v[0] = q.x; r.v[1] = q.y;
-  } else {
-    r.v[0] = *reinterpret_cast<const uint32_t*>(p);
-  }
-  return r;
-}
-
-template <int PREC, int C>
-__device__ __forceinline__ void store_cells(typename Store<PREC>::T* __restrict__ p, const Cells<PREC, C>& r) {
-  if constexpr (Cells<PREC, C>::N == 4) *reinterpret_cast<uint4*>(p) = make_uint4(r.v[0], r.v[1], r.v[2], r.v[3]);
-  else if constexpr (Cells<PREC, C>::N == 2) *reinterpret_cast<uint2*>(p) = make_uint2(r.v[0], r.v[1]);
-  else *reinterpret_cast<uint32_t*>(p) = r.v[0];
-}
-
-// cell c in true units
-template <int PREC, int C>
-__device__ __forceinline__ float get_cell(const Cells<PREC, C>& r, int c, float inv) {
-  if constexpr (PREC == PREC_FP32) {
-    return __uint_as_float(r.v[c]);
-  } else {
-    const float2 p = Store<PREC>::w2f(r.v[c >> 1]);
-    return ((c & 1) ? p.y : p.x) * inv;
-  }
-}
-
-// bits of one stored value
-template <int PREC>
-__device__ __forceinline__ uint32_t raw_bits(const typename Store<PREC>::T* p) {
-  if constexpr (PREC == PREC_FP32) return __float_as_uint(*p);
-  else return Store<PREC>::bits(*p);
-}
-
-template <int PREC, int C>
-__device__ __forceinline__ void put_bits(Cells<PREC, C>& r, int c, uint32_t b) {
-  if constexpr (PREC == PREC_FP32) r.v[c] = b;
-  else r.v[c >> 1] = (c & 1) ? __byte_perm(r.v[c >> 1], b, 0x5410) : __byte_perm(b, r.v[c >> 1], 0x7610);
-}
-
-template <int PREC, int C>
-__device__ __forceinline__ void put_cell(Cells<PREC, C>& r, int c, float v, float sc) {
-  if constexpr (PREC == PREC_FP32) {
-    r.v[c] = __float_as_uint(v);
-  } else {
-    const typename Store<PREC>::T e = Store<PREC>::enc(v, sc);
-    put_bits<PREC, C>(r, c, Store<PREC>::bits(e));
-  }
-}
-
-// bits of cell c
-template <int PREC, int C>
-__device__ __forceinline__ uint32_t cell_bits(const Cells<PREC, C>& r, int c) {
-  if constexpr (PREC == PREC_FP32) return r.v[c];
-  else return (c & 1) ? r.v[c >> 1] >> 16 : r.v[c >> 1] & 0xffffu;
-}
-
-// one stored value in true units
-template <int PREC>
-__device__ __forceinline__ float true_value(uint32_t bits, float inv) {
-  if constexpr (PREC == PREC_FP32) return __uint_as_float(bits);
-  else return Store<PREC>::w2f(bits).x * inv;
-}
-
-// the cells x - SH of the row whose cells x a warp holds (the first / last lane's outer cell repeats its own)
-template <int PREC, int C, int SH>
-__device__ __forceinline__ Cells<PREC, C> shift_cells(const Cells<PREC, C>& r) {
-  constexpr int N = Cells<PREC, C>::N;
-  Cells<PREC, C> o;
-  if constexpr (SH == 0) {
-    o = r;
-  } else if constexpr (SH == 1) {
-    const uint32_t l = __shfl_up_sync(kFull, r.v[N - 1], 1);
-#pragma unroll
-    for (int k = N - 1; k >= 0; --k) {
-      const uint32_t below = k ? r.v[k - 1] : l;
-      o.v[k] = PREC == PREC_FP32 ? below : __byte_perm(below, r.v[k], 0x5432);
-    }
-  } else {
-    const uint32_t g = __shfl_down_sync(kFull, r.v[0], 1);
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const uint32_t above = k < N - 1 ? r.v[k + 1] : g;
-      o.v[k] = PREC == PREC_FP32 ? above : __byte_perm(r.v[k], above, 0x5432);
-    }
-  }
-  return o;
-}
 
 // Strips and segments of one lattice (see k_march).
 struct March {
@@ -156,27 +52,27 @@ __host__ __device__ inline int march_x0(int strip, bool wrap) {
   return strip * march_out<PREC, C>(wrap) - (wrap ? march_halo<PREC, C>(true) * C : 0);
 }
 
-__device__ __forceinline__ void copy_async16(void* smem, const void* gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void copy_async8(void* smem, const void* gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void copy_async4(void* smem, const void* gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // One warp's march over the rows [ya, yb) of a strip.  XE: the strip has an x side (or, with 16-bit
 // storage, a frame group) within reach; YE: the rows have a y side within reach.
 template <int PREC, bool HET, bool THERMAL, int C, int STAGES, bool XE, bool YE>
-struct Marcher {
-  using S = Store<PREC>;
-  using E = typename S::T;
-  using V = Cells<PREC, C>;
-  static constexpr bool EDGE = XE || YE;
+struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE> {
+  using Ops = RowOps<PREC, HET, THERMAL, C, XE, YE>;
+  using typename Ops::E;
+  using typename Ops::V;
+  using Ops::EDGE;
+  using Ops::P;
+  using Ops::lane;
+  using Ops::x0;
+  using Ops::slow;
+  using Ops::left;
+  using Ops::right;
+  using Ops::wrap_y;
+  using Ops::low;
+  using Ops::high;
+  using Ops::col;
+  using Ops::shift;
+  using Ops::collide_row;
+  using Ops::pick;
   static constexpr int kPlanes = THERMAL ? 13 : 8;
   static constexpr int kRow = 32 * C * (int)sizeof(E);      // bytes of a plane's row
   static constexpr int kMed = 32 * C * (int)sizeof(float);  // bytes of a medium field's row
@@ -184,32 +80,13 @@ struct Marcher {
   static constexpr int kChunks = kRow / 16, kMedChunks = kMed / 16;
   static constexpr int kCopies = (kPlanes * kChunks + 31) / 32;
 
-  const StepParams& P;
   char* buf;     // the warp's STAGES stages in shared memory
-  int lane, xs;  // xs: column of the warp's first cell
-  int x0;        // (unwrapped) column of the lane's first cell
+  int xs;        // column of the warp's first cell
   bool out;      // the lane stores its cells
-  // XE only
-  bool slow;            // (uniform) the strip crosses a periodic side
-  bool left, right;     // the lane holds the first / last column, between walls
-  bool frame;           // 16-bit storage: the lane's cells are a frame group of k_step, which takes the FP32 collision
-  int cr;               // component of the last column
-  float dot[3];         // e_i . u_w of the side wall of the lane's first / last column
   uint32_t at[kCopies]; // (EDGE: unused)
-  uint32_t e[3], eg;    // own populations of that column that bounce back there, of the row loaded next
+  uint32_t e[3], eg;    // XE: own populations of the lane's side column that bounce back there, of the row loaded next
 
-  __device__ __forceinline__ Marcher(const StepParams& p, char* b) : P(p), buf(b) {}
-
-  __device__ __forceinline__ int wrap_x(int x) const { return x < 0 ? x + P.nx : (x >= P.nx ? x - P.nx : x); }
-  __device__ __forceinline__ int wrap_y(int y) const { return !YE ? y : y < 0 ? y + P.ny : (y >= P.ny ? y - P.ny : y); }
-  __device__ __forceinline__ bool low(int y) const { return YE && P.bc_y == BC_WALL && y == 0; }
-  __device__ __forceinline__ bool high(int y) const { return YE && P.bc_y == BC_WALL && y == P.ny - 1; }
-  // column of the lane's cell c in memory (clamped where the cell is never part of a stored result)
-  __device__ __forceinline__ int col(int c) const {
-    if constexpr (!XE) return x0 + c;
-    const int x = slow ? wrap_x(x0 + c) : x0 + c;
-    return x < P.nx ? x : P.nx - 1;
-  }
+  __device__ __forceinline__ Marcher(const StepParams& p, char* b) : Ops(p), buf(b) {}
 
   // Start of plane p's row that the pull into row y (in memory) reads.  At a wall row the populations
   // that come through the wall are the row's own opposite ones.
@@ -319,201 +196,6 @@ struct Marcher {
     }
   }
 
-  // the one-cell x shifts of the pull into row y (none for populations that came back from a wall row)
-  __device__ __forceinline__ void shift(int y, V f[8], V g[5]) const {
-    f[0] = shift_cells<PREC, C, 1>(f[0]);
-    f[2] = shift_cells<PREC, C, -1>(f[2]);
-    if (!low(y)) {
-      f[4] = shift_cells<PREC, C, 1>(f[4]);
-      f[5] = shift_cells<PREC, C, -1>(f[5]);
-    }
-    if (!high(y)) {
-      f[6] = shift_cells<PREC, C, -1>(f[6]);
-      f[7] = shift_cells<PREC, C, 1>(f[7]);
-    }
-    if constexpr (THERMAL) {
-      g[1] = shift_cells<PREC, C, 1>(g[1]);
-      g[3] = shift_cells<PREC, C, -1>(g[3]);
-    }
-  }
-
-  // One cell in true units with its wall links patched: d, g pulled (wall links: the own opposite population).
-  __device__ __forceinline__ void patch_cell(int c, int y, const uint32_t e[3], uint32_t eg, float d[8], float g[5]) const {
-    const bool lo = low(y), hi = high(y);
-    if (lo) {
-      d[1] = bounce<PREC>(P, d[1], 1, wall_dot(P, 1, 2));
-      d[4] = bounce<PREC>(P, d[4], 4, wall_dot(P, 4, 2));
-      d[5] = bounce<PREC>(P, d[5], 5, wall_dot(P, 5, 2));
-      if constexpr (THERMAL) g[2] = heat_bounce<PREC>(P, g[2], 2);
-    }
-    if (hi) {
-      d[3] = bounce<PREC>(P, d[3], 3, wall_dot(P, 3, 3));
-      d[6] = bounce<PREC>(P, d[6], 6, wall_dot(P, 6, 3));
-      d[7] = bounce<PREC>(P, d[7], 7, wall_dot(P, 7, 3));
-      if constexpr (THERMAL) g[4] = heat_bounce<PREC>(P, g[4], 3);
-    }
-    if constexpr (XE) {
-      const float inv = P.inv_scale;
-      if (left && c == 0) {
-        d[0] = bounce<PREC>(P, true_value<PREC>(e[0], inv), 0, dot[0]);
-        if (!lo) d[4] = bounce<PREC>(P, true_value<PREC>(e[1], inv), 4, dot[1]);
-        if (!hi) d[7] = bounce<PREC>(P, true_value<PREC>(e[2], inv), 7, dot[2]);
-        if constexpr (THERMAL) g[1] = heat_bounce<PREC>(P, true_value<PREC>(eg, inv), 0);
-      }
-      if (right && c == cr) {
-        d[2] = bounce<PREC>(P, true_value<PREC>(e[0], inv), 2, dot[0]);
-        if (!lo) d[5] = bounce<PREC>(P, true_value<PREC>(e[1], inv), 5, dot[1]);
-        if (!hi) d[6] = bounce<PREC>(P, true_value<PREC>(e[2], inv), 6, dot[2]);
-        if constexpr (THERMAL) g[3] = heat_bounce<PREC>(P, true_value<PREC>(eg, inv), 1);
-      }
-    }
-  }
-
-  // The FP32 collision of the lane's cells of row y, in place, wall links first.
-  __device__ __forceinline__ float collide_edge(int y, const float ph[], const float k[], const uint32_t e[3], uint32_t eg, V w[8],
-                                                V gw[5]) const {
-    float check = 0.0f;
-#pragma unroll
-      for (int h = 0; h < C / 2; ++h) {
-        const int ca = 2 * h, cb = ca + 1;
-        float da[8], db[8], ga[5], gb[5];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          da[i] = get_cell<PREC, C>(w[i], ca, P.inv_scale);
-          db[i] = get_cell<PREC, C>(w[i], cb, P.inv_scale);
-        }
-        if constexpr (THERMAL) {
-#pragma unroll
-          for (int i = 0; i < 5; ++i) {
-            ga[i] = get_cell<PREC, C>(gw[i], ca, P.inv_scale);
-            gb[i] = get_cell<PREC, C>(gw[i], cb, P.inv_scale);
-          }
-        }
-        patch_cell(ca, y, e, eg, da, ga);
-        patch_cell(cb, y, e, eg, db, gb);
-        PairMedium m;
-        if constexpr (HET) {
-          const float* sv = P.sv ? P.sv + (int64_t)y * P.pitch : nullptr;
-          m = pair_medium(coef_of(P, ph[ca], k[ca], sv ? __ldg(sv + col(ca)) : P.s_v), coef_of(P, ph[cb], k[cb], sv ? __ldg(sv + col(cb)) : P.s_v));
-        } else {
-          m = pair_medium(coef_uniform(P), coef_uniform(P));
-        }
-        float2 d[8], g[5], n0, ay = f2(P.ay), ux, uy;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) d[i] = make_float2(da[i], db[i]);
-        if constexpr (THERMAL) {
-#pragma unroll
-          for (int i = 0; i < 5; ++i) g[i] = make_float2(ga[i], gb[i]);
-          n0 = add2(add2(add2(add2(g[0], g[1]), g[2]), g[3]), g[4]);
-          ay = fma2(f2(P.g_beta), n0, ay);  // a = g beta (T - T0) j
-        }
-        collide_d2q8_pair(d, m, P.ax, ay, P, ux, uy);
-        check += (fabsf(ux.x) + fabsf(uy.x)) + (fabsf(ux.y) + fabsf(uy.y));
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          put_cell<PREC, C>(w[i], ca, d[i].x, P.scale);
-          put_cell<PREC, C>(w[i], cb, d[i].y, P.scale);
-        }
-        if constexpr (THERMAL) {
-          collide_d2q5_pair_fp32(g, n0, ux, uy, P);
-#pragma unroll
-          for (int i = 0; i < 5; ++i) {
-            put_cell<PREC, C>(gw[i], ca, g[i].x, P.scale);
-            put_cell<PREC, C>(gw[i], cb, g[i].y, P.scale);
-          }
-        }
-      }
-    return check;
-  }
-
-  // viscous rates of the lane's cells a, a + 1 of row y
-  __device__ __forceinline__ float2 rates(int y, int a) const {
-    const float* sv = P.sv + (int64_t)y * P.pitch;
-    return make_float2(__ldg(sv + col(a)), __ldg(sv + col(a + 1)));
-  }
-
-  // Collision of the lane's cells of row y, in place; returns the sum of |u| over the cells.
-  __device__ __forceinline__ float collide(int y, const float ph[], const float k[], V w[8], V gw[5]) const {
-    float check = 0.0f;
-    if constexpr (PREC == PREC_FP32) {
-#pragma unroll
-      for (int h = 0; h < C / 2; ++h) {
-        const int a = 2 * h, b = a + 1;
-        float2 d[8], ux, uy, ay = f2(P.ay);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) d[i] = make_float2(__uint_as_float(w[i].v[a]), __uint_as_float(w[i].v[b]));
-        PairMedium m;
-        if constexpr (HET) {
-          const float2 sv = P.sv ? rates(y, a) : f2(P.s_v);
-          m = pair_medium(coef_of(P, ph[a], k[a], sv.x), coef_of(P, ph[b], k[b], sv.y));
-        } else {
-          m = pair_medium(coef_uniform(P), coef_uniform(P));
-        }
-        float2 g[5], n0;
-        if constexpr (THERMAL) {
-#pragma unroll
-          for (int i = 0; i < 5; ++i) g[i] = make_float2(__uint_as_float(gw[i].v[a]), __uint_as_float(gw[i].v[b]));
-          n0 = add2(add2(add2(add2(g[0], g[1]), g[2]), g[3]), g[4]);
-          ay = fma2(f2(P.g_beta), n0, ay);  // a = g beta (T - T0) j
-        }
-        collide_d2q8_pair(d, m, P.ax, ay, P, ux, uy);
-        check += (fabsf(ux.x) + fabsf(uy.x)) + (fabsf(ux.y) + fabsf(uy.y));
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { w[i].v[a] = __float_as_uint(d[i].x); w[i].v[b] = __float_as_uint(d[i].y); }
-        if constexpr (THERMAL) {
-          collide_d2q5_pair_fp32(g, n0, ux, uy, P);
-#pragma unroll
-          for (int i = 0; i < 5; ++i) { gw[i].v[a] = __float_as_uint(g[i].x); gw[i].v[b] = __float_as_uint(g[i].y); }
-        }
-      }
-    } else {
-#pragma unroll
-      for (int h = 0; h < C / 2; ++h) {
-        float2 dp[8], ux, uy;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) dp[i] = S::w2f(w[i].v[h]);
-        if constexpr (HET) {
-          float2 hx, hy;
-          const float2 sv = P.sv ? rates(y, 2 * h) : f2(P.s_v);
-          const PairCoef c = pair_coef_het(P, make_float2(ph[2 * h], ph[2 * h + 1]), make_float2(k[2 * h], k[2 * h + 1]), sv, hx, hy);
-          collide_pair(dp, c, hx, hy, P.pc, ux, uy);
-        } else if constexpr (THERMAL) {
-          float2 gp[5];
-#pragma unroll
-          for (int i = 0; i < 5; ++i) gp[i] = S::w2f(gw[i].v[h]);
-          const float2 sTd = add2(add2(add2(gp[0], gp[1]), add2(gp[2], gp[3])), gp[4]);  // s (T - T0)
-          const float2 hy = mul2(f2(P.phi_u), fma2(f2(0.5f * P.g_beta * P.inv_scale), sTd, f2(P.pc.hay)));
-          collide_pair(dp, pair_coef_uniform(P.pc), f2(P.pc.u_hx), hy, P.pc, ux, uy);
-          collide_d2q5_pair(gp, ux, uy, P);
-#pragma unroll
-          for (int i = 0; i < 5; ++i) gw[i].v[h] = S::f2w(gp[i]);
-        } else {
-          collide_pair(dp, pair_coef_uniform(P.pc), f2(P.pc.u_hx), f2(P.pc.u_hy), P.pc, ux, uy);
-        }
-        check += (fabsf(ux.x) + fabsf(uy.x)) + (fabsf(ux.y) + fabsf(uy.y));
-#pragma unroll
-        for (int i = 0; i < 8; ++i) w[i].v[h] = S::f2w(dp[i]);
-      }
-    }
-    return check;
-  }
-
-  __device__ __forceinline__ float collide_row(int y, const float ph[], const float k[], const uint32_t e[3], uint32_t eg, V w[8],
-                                               V gw[5]) const {
-    if constexpr (EDGE) {
-      if (PREC == PREC_FP32 || frame || low(y) || high(y)) return collide_edge(y, ph, k, e, eg, w, gw);
-    }
-    return collide(y, ph, k, w, gw);
-  }
-
-  // bits of component cr
-  __device__ __forceinline__ uint32_t pick(const V& v) const {
-    uint32_t r = cell_bits<PREC, C>(v, 0);
-#pragma unroll
-    for (int c = 1; c < C; ++c) r = cr == c ? cell_bits<PREC, C>(v, c) : r;
-    return r;
-  }
-
   __device__ __forceinline__ void store(int y, V w[8], V gw[5]) const {
     if (XE && x0 + C > P.nx) {  // row padding holds zeros
 #pragma unroll
@@ -543,29 +225,11 @@ struct Marcher {
   }
 
   __device__ __forceinline__ void run(const March& M, int strip, int ya, int yb) {
-    lane = threadIdx.x & 31;
     xs = march_x0<PREC, C>(strip, M.wrap);
-    x0 = xs + lane * C;
+    Ops::set_lane(xs, M.wrap);
     const int halo = march_halo<PREC, C>(M.wrap);
-    if constexpr (!XE) {
-      out = lane >= halo && lane < 32 - halo;
-    } else {
-      const int nx = P.nx;
-      const bool first = !M.wrap && strip == 0, last = !M.wrap && strip == M.strips - 1;
-      out = (lane >= halo || first) && (lane < 32 - halo || last) && x0 < nx;
-      slow = M.wrap && (xs < 0 || xs + 32 * C > nx);
-      left = P.bc_x == BC_WALL && x0 == 0;
-      right = P.bc_x == BC_WALL && x0 <= nx - 1 && x0 + C > nx - 1;
-      cr = (nx - 1) & (C - 1);
-      frame = PREC != PREC_FP32 && (x0 < 4 || x0 + C > (nx - 1) / 4 * 4);
-      if (left || right) {
-        const int w = left ? 0 : 1;
-        dot[0] = left ? wall_dot(P, 0, w) : wall_dot(P, 2, w);
-        dot[1] = left ? wall_dot(P, 4, w) : wall_dot(P, 5, w);
-        dot[2] = left ? wall_dot(P, 7, w) : wall_dot(P, 6, w);
-      }
-    }
-    if constexpr (EDGE && !XE) frame = false;
+    const bool first = XE && !M.wrap && strip == 0, last = XE && !M.wrap && strip == M.strips - 1;
+    out = (lane >= halo || first) && (lane < 32 - halo || last) && (!XE || x0 < P.nx);
     const bool walls = YE && P.bc_y == BC_WALL;
     const int lo = walls && ya == 0 ? 0 : ya - 1, hi = walls && yb == P.ny ? yb : yb + 1;  // rows of the first step
     float check = 0.0f;
@@ -674,9 +338,6 @@ struct Marcher {
   }
 };
 
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // The warps at the sides: the bottom and top segments, then the strips with an x side in pieces of
 // `rows` rows.  A kernel of its own, so that the rules at the sides cost the main one no registers;
 // it lets the main kernel start at once (the two write different cells).
@@ -738,7 +399,7 @@ bool march_takes(const StepParams& P, int prec, bool het, bool thermal) {
   return true;
 }
 
-static int sm_count() {
+int sm_count() {
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
     cudaGetLastError();
