@@ -277,6 +277,8 @@ __device__ __forceinline__ float group8_sum(float v, unsigned mask) {
 template <int PREC, bool HET>
 __global__ void k_adj_nee(const StepParams P, const void* buf, float* __restrict__ nu, float* __restrict__ g_l,
                           float* __restrict__ g_phi) {
+  launch_dependents();
+  wait_prerequisites();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int grp = t >> 3, i = t & 7;
   const bool shared_nb = P.nx < 4;
@@ -597,6 +599,8 @@ __device__ __forceinline__ void adj_item(const StepParams& P, const void* buf, c
 #endif
 template <int PREC, bool HET>
 __global__ void __launch_bounds__(kStepThreads, LBM_ADJ_MIN_CTAS) k_adj_step(const StepParams P, const void* buf, AdjArgs A, AdjTiling tl) {
+  launch_dependents();
+  wait_prerequisites();
   adj_item<PREC, HET, kStepThreads>(P, buf, A, tl, blockIdx.x);
 }
 
@@ -656,7 +660,7 @@ cudaError_t launch_adj_nee(const StepParams& P, int prec, bool het, const void* 
                            cudaStream_t s) {
   const int threads = 8 * (P.nx < 4 ? P.ny : 2 * P.ny);
   const int blocks = (threads + 127) / 128;
-#define CALL_NEE(PR, H) k_adj_nee<PR, H><<<blocks, 128, 0, s>>>(P, buf, nu, g_l, g_phi)
+#define CALL_NEE(PR, H) return launch_early(k_adj_nee<PR, H>, dim3(blocks), dim3(128), 0, s, P, buf, nu, g_l, g_phi)
   LBM_ADJ_DISPATCH(prec, het, CALL_NEE);
 #undef CALL_NEE
   return cudaGetLastError();
@@ -679,7 +683,7 @@ cudaError_t launch_adj_step(const StepParams& P, int prec, bool het, const void*
   AdjArgs A{nu_in, nu_out, g_l, g_phi};
   const AdjTiling tl = adj_tiling_of(P.nx, P.ny, P.bc_y, kStepThreads);
   const unsigned blocks = (unsigned)((long long)tl.frame_blocks + adj_main_items(tl, P.ny));
-#define CALL_ADJ(PR, H) k_adj_step<PR, H><<<blocks, kStepThreads, 0, s>>>(P, buf, A, tl)
+#define CALL_ADJ(PR, H) return launch_early(k_adj_step<PR, H>, dim3(blocks), dim3(kStepThreads), 0, s, P, buf, A, tl)
   LBM_ADJ_DISPATCH(prec, het, CALL_ADJ);
 #undef CALL_ADJ
   return cudaGetLastError();

@@ -239,6 +239,8 @@ __global__ void k_macros(const StepParams P, float* __restrict__ p, float* __res
 // one cell's (p, ux, uy, T) into out[0..3] (T = 0 without a temperature field)
 template <int PREC, bool HET, bool THERMAL>
 __global__ void k_probe(const StepParams P, int x, int y, float* __restrict__ out) {
+  launch_dependents();
+  wait_prerequisites();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   float d[8], gd[5], ay;
   gather_state<PREC, HET, THERMAL>(P, P.src, P.gsrc, x, y, d, gd, ay);
@@ -437,17 +439,18 @@ cudaError_t launch_macros(const StepParams& P, int prec, bool het, bool thermal,
 
 // a few floats, e.g. wall velocities from page-locked host memory that the device reads directly
 __global__ void k_copy_small(float* __restrict__ dst, const float* __restrict__ src, int n) {
+  launch_dependents();
+  wait_prerequisites();
   const int i = threadIdx.x;
   if (i < n) dst[i] = src[i];
 }
 
 cudaError_t launch_copy_small(float* dst, const float* src, int n, cudaStream_t s) {
-  k_copy_small<<<1, 32, 0, s>>>(dst, src, n);
-  return cudaGetLastError();
+  return launch_early(k_copy_small, dim3(1), dim3(32), 0, s, dst, src, n);
 }
 
 cudaError_t launch_probe(const StepParams& P, int prec, bool het, bool thermal, int x, int y, float* out, cudaStream_t s) {
-#define CALL_PROBE(PR, H, TH) k_probe<PR, H, TH><<<1, 32, 0, s>>>(P, x, y, out)
+#define CALL_PROBE(PR, H, TH) return launch_early(k_probe<PR, H, TH>, dim3(1), dim3(32), 0, s, P, x, y, out)
   LBM_DISPATCH_PHT(prec, het, thermal, CALL_PROBE);
 #undef CALL_PROBE
   return cudaGetLastError();

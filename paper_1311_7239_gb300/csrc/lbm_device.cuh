@@ -86,6 +86,12 @@ __device__ __forceinline__ bool dbg_check(const StepParams& P, bool ok) {
 #endif
 }
 
+// Programmatic dependent launch: the kernels of a step sequence let the next one on the stream be
+// launched while they still run, and touch memory only after the one before has ended, which hides
+// the launch latency (launch_early on the host).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // D2Q8 velocities of Eq. 7 and the weights w_i listed after Eq. 20 (w_1..4 = 1/9, w_5..8 = 1/36).
 __device__ __forceinline__ int ex_of(int i) { return (i == 0 || i == 4 || i == 7) ? 1 : ((i == 2 || i == 5 || i == 6) ? -1 : 0); }
 __device__ __forceinline__ int ey_of(int i) { return (i == 1 || i == 4 || i == 5) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0); }
@@ -812,18 +818,34 @@ __device__ __forceinline__ void pull_cell_g(const StepParams& P, const typename 
 // Non-equilibrium extrapolation of a pressure column: replaces d of the cell (xb, y) by
 // f_eq(p_b, u_nb; phi_b) + f_nb - f_eq(p_nb, u_nb; phi_nb) with nb = (xb +- 1, y), in deviations.
 // (dn: the pulled state of nb)
+// The multiply-adds are written out, so that every kernel extrapolates to the same bits (macro_d2q8
+// and feq_dev_d2q8, which leave them to the compiler, serve the read-outs).
+// (cn, cb: the medium of the inner neighbour and of the column's cell, pb its pressure)
+__device__ __forceinline__ void pressure_cell(const StepParams& P, const float dn[8], const Coef& cn, const Coef& cb, float pb, float d[8]) {
+  const float m1 = dn[0] + dn[1] + dn[2] + dn[3] + dn[4] + dn[5] + dn[6] + dn[7];
+  const float jx = (dn[0] - dn[2]) + (dn[4] - dn[5] - dn[6] + dn[7]);
+  const float jy = (dn[1] - dn[3]) + (dn[4] + dn[5] - dn[6] - dn[7]);
+  const float h = 0.5f * cn.phi, inv_rho0 = fast_rcp(P.rho0);
+  const float vx = __fmaf_rn(h, P.ax, __fmul_rn(jx, inv_rho0)), vy = __fmaf_rn(h, P.ay, __fmul_rn(jy, inv_rho0));
+  const float l0 = __fmaf_rn(0.25f, cn.c_lin, 0.5f);
+  const float R = __fmaf_rn(l0, l0, __fmul_rn(0.5f * cn.c_nl, fast_sqrt(__fmaf_rn(vx, vx, __fmul_rn(vy, vy)))));
+  const float inv = rcp_normal(__fadd_rn(l0, __fmul_rn(R, rsqrt_normal(R))));
+  const float ux = vx * inv, uy = vy * inv, usq = __fmaf_rn(ux, ux, __fmul_rn(uy, uy));
+  const float pn = 0.6f * __fmaf_rn(-__fmul_rn((2.0f / 3.0f) * P.rho0, usq), cn.inv_phi, m1);  // phi p - p_rest, Eq. 20
+  const float pd = __fmaf_rn(cb.phi, pb, -P.p_rest);
+  const float ub = __fmul_rn(1.5f * usq, cb.inv_phi), un = __fmul_rn(1.5f * usq, cn.inv_phi);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {  // f_eq of Eq. 22 in deviations
+    const float eu = __fadd_rn((float)ex_of(i) * ux, (float)ey_of(i) * uy), q = __fmul_rn(4.5f * eu, eu);
+    const float eb = __fmul_rn(w_of(i), __fmaf_rn(3.0f, pd, __fmul_rn(P.rho0, __fmaf_rn(3.0f, eu, __fmaf_rn(q, cb.inv_phi, -ub)))));
+    const float en = __fmul_rn(w_of(i), __fmaf_rn(3.0f, pn, __fmul_rn(P.rho0, __fmaf_rn(3.0f, eu, __fmaf_rn(q, cn.inv_phi, -un)))));
+    d[i] = __fadd_rn(__fadd_rn(eb, dn[i]), -en);
+  }
+}
+
 template <bool HET>
 __device__ __forceinline__ void pressure_column_from(const StepParams& P, const float dn[8], int xb, int y, float d[8]) {
-  const int xn = xb == 0 ? 1 : P.nx - 2;
-  const float pb = xb == 0 ? P.p_in : P.p_out;
-  const Coef cn = coef_at<HET>(P, xn, y);
-  const Coef cb = coef_at<HET>(P, xb, y);
-  const Macro mn = macro_d2q8(dn, cn, P.ax, P.ay, P.rho0);
-  float eb[8], en[8];
-  feq_dev_d2q8(cb.phi * pb - P.p_rest, mn.ux, mn.uy, cb.inv_phi, P.rho0, eb);
-  feq_dev_d2q8(mn.phip_dev, mn.ux, mn.uy, cn.inv_phi, P.rho0, en);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) d[i] = eb[i] + dn[i] - en[i];
+  pressure_cell(P, dn, coef_at<HET>(P, xb == 0 ? 1 : P.nx - 2, y), coef_at<HET>(P, xb, y), xb == 0 ? P.p_in : P.p_out, d);
 }
 
 template <int PREC, bool HET>

@@ -11,6 +11,23 @@ namespace lbm {
 constexpr int kResidualMaxBlocks = 2048;  // partial-sum slots of the residual reduction
 
 int record_error(int code, const char* msg);
+
+// Launch of a kernel that begins with wait_prerequisites(): it may be scheduled while the kernel
+// before it on the stream still runs.
+template <class... P, class... A>
+inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
 }  // namespace lbm
 struct lbm_config;
 namespace lbm {

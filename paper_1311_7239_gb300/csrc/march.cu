@@ -381,18 +381,21 @@ __global__ void __launch_bounds__(kMarchThreads, CTAS) k_march(const __grid_cons
   wait_prerequisites();
 }
 
-// Which contexts take their steps in pairs.  Periodic and halfway-wall sides; with 16-bit storage and
+// Which contexts take their steps in pairs.  Periodic and halfway-wall sides, and with FP32 storage
+// pressure columns; with 16-bit storage and
 // periodic x sides the halo must be whole groups of four cells (k_step's frame groups round
 // differently).  Below the size of L2 (129 MB) single steps do not go to HBM and their many small
 // warps win: 1024^2 FP32 8.6 us per step against 9.8 in pairs, 1536^2 24.6 against 17.0; with
 // temperature 1024^2 (109 MB) 16.5 against 11.6.  16-bit storage is bound by the collisions rather
-// than by HBM, and gains only where the state is several times L2.
+// than by HBM: the uniform medium gains from the size of L2 on (2048^2 FP16 26.3 -> 24.0 us, 1536^2
+// 13.4 -> 15.7), a per-cell medium or the temperature does not (4096^2 per-cell 111 -> 114, 2048^2
+// temperature 40.8 -> 45.5).
 bool march_takes(const StepParams& P, int prec, bool het, bool thermal) {
   const uint64_t bytes = 2 * (uint64_t)(thermal ? 13 : 8) * (uint64_t)P.nx * P.ny * (prec == PREC_FP32 ? 4 : 2);
-  if (bytes < (prec == PREC_FP32 ? 100ull << 20 : 400ull << 20)) return false;
+  if (bytes < (prec == PREC_FP32 ? 100ull << 20 : 120ull << 20)) return false;
   if (prec != PREC_FP32 && (het || thermal)) return false;
   if (P.inplace || P.nx < 16 || P.ny < 16) return false;
-  if (P.bc_x > BC_WALL || P.bc_y > BC_WALL) return false;
+  if (P.bc_x > BC_PRESSURE || P.bc_y > BC_WALL || (P.bc_x == BC_PRESSURE && (prec != PREC_FP32 || thermal))) return false;
   if (P.bc_x == BC_PERIODIC && prec != PREC_FP32 && (P.nx & 3)) return false;
   if (het && thermal) return false;
   if (8 * (uint64_t)P.plane * (prec == PREC_FP32 ? 4 : 2) / 16 >= (1ull << 32)) return false;  // (fill's 32-bit offsets)
@@ -413,14 +416,13 @@ static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
   March M;
   M.wrap = P.bc_x == BC_PERIODIC;
   M.strips = march_strips<PREC, C>(P.nx, M.wrap);
-  // sides: short segments, whose warps are done before the main kernel's
-  M.side_rows = 8;
   auto xs = [&](int k) { return march_x0<PREC, C>(k, M.wrap); };
   auto inner_strip = [&](int k) { return xs(k) >= 4 && xs(k) + 32 * C <= (P.nx - 1) / 4 * 4; };
   for (M.s0 = 0; M.s0 < M.strips && !inner_strip(M.s0);) ++M.s0;
   for (M.s1 = M.s0; M.s1 < M.strips && inner_strip(M.s1);) ++M.s1;
-  // rows per segment: whole waves of resident warps, at most 24 rows (longer segments drift apart and
-  // lose the halo columns from L2: 4096^2 FP32 93.5 us at 25 rows, 102 at 50), at least 12
+  // Rows per segment: whole waves of resident warps, at most 24 rows (longer segments drift apart and
+  // lose the halo columns from L2: 4096^2 FP32 93.5 us at 25 rows, 102 at 50), at least 12.  The strips
+  // at the sides, whose warps are slower, take short segments.
   const int ny = P.ny - 2 * kMarchSide, strips = M.s1 - M.s0 > 0 ? M.s1 - M.s0 : 1;
   const int64_t resident = (int64_t)sm_count() * CTAS * (kMarchThreads / 32);
   M.rows = ny;
@@ -429,6 +431,7 @@ static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
     if (segs > 0) M.rows = (int)((ny + segs - 1) / segs);
   }
   if (M.rows < 12) M.rows = 12;
+  M.side_rows = 8;
   M.segs = (ny + M.rows - 1) / M.rows;
   M.side_segs = (ny + M.side_rows - 1) / M.side_rows;
   const size_t bytes = (kMarchThreads / 32) * STAGES * Marcher<PREC, HET, THERMAL, C, STAGES, false, false>::kStage;
@@ -439,21 +442,9 @@ static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const int side_items = 2 * M.strips + (M.strips - (M.s1 - M.s0)) * M.side_segs;
   side<<<(side_items + 3) / 4, kMarchThreads, bytes, s>>>(P, M);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int items = (M.s1 - M.s0) * M.segs;
-  if (items > 0) {
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3((items + 3) / 4);
-    c.blockDim = dim3(kMarchThreads);
-    c.dynamicSmemBytes = bytes;
-    c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = 1;
-    e = cudaLaunchKernelEx(&c, main, P, M);
-    if (e != cudaSuccess) return e;
-  }
+  if (items > 0 && (e = launch_early(main, dim3((items + 3) / 4), dim3(kMarchThreads), bytes, s, P, M)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

@@ -123,9 +123,6 @@ __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_gr
 template <int N>
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // The rules of one row for a warp whose lane holds the cells x0 .. x0 + C - 1.  XE: the warp's cells have
 // an x side (or, with 16-bit storage, a frame group) within reach; YE: the rows a y side.
 template <int PREC, bool HET, bool THERMAL, int C, bool XE, bool YE>
@@ -134,6 +131,7 @@ struct RowOps {
   using E = typename S::T;
   using V = Cells<PREC, C>;
   static constexpr bool EDGE = XE || YE;
+  static constexpr bool kPressure = XE && PREC == PREC_FP32 && !THERMAL;
 
   const StepParams& P;
   int lane, x0;         // (unwrapped) column of the lane's first cell
@@ -141,6 +139,7 @@ struct RowOps {
   bool slow;            // (uniform) the warp's cells cross a periodic side
   bool left, right;     // the lane holds the first / last column, between walls
   bool any_left, any_right;  // (uniform) one of the warp's lanes does
+  bool inlet, outlet;        // the lane holds a pressure column, x = 0 or nx - 1 (FP32 storage)
   bool frame;           // 16-bit storage: the lane's cells are a frame group of k_step, which takes the FP32 collision
   int cr;               // component of the last column
   float dot[3];         // e_i . u_w of the side wall of the lane's first / last column
@@ -159,6 +158,8 @@ struct RowOps {
       right = P.bc_x == BC_WALL && x0 <= nx - 1 && x0 + C > nx - 1;
       any_left = P.bc_x == BC_WALL && xs <= 0;
       any_right = P.bc_x == BC_WALL && xs + 32 * C > nx - 1;
+      inlet = kPressure && P.bc_x == BC_PRESSURE && x0 == 0;
+      outlet = kPressure && P.bc_x == BC_PRESSURE && x0 <= nx - 1 && x0 + C > nx - 1;
       cr = (nx - 1) & (C - 1);
       frame = PREC != PREC_FP32 && frame_cells();
       dot[0] = dot[1] = dot[2] = 0.0f;
@@ -254,6 +255,28 @@ struct RowOps {
   __device__ __forceinline__ float collide_edge(int y, const float ph[], const float k[], const uint32_t e[3], uint32_t eg, V w[8],
                                                 V gw[5]) const {
     float check = 0.0f;
+    // Pressure columns are extrapolated from the pulled state of their inner neighbour.  Where the last
+    // column is the first cell of a pair, that neighbour is in the pair or the lane before.
+    float inner[8], inner_ph = 0.0f, inner_k = 0.0f;
+    if constexpr (kPressure) {
+      if (P.bc_x == BC_PRESSURE && (cr & 1) == 0) {
+        float unused[5];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float before = __shfl_up_sync(kFull, get_cell<PREC, C>(w[i], C - 1, 1.0f), 1);
+          inner[i] = C == 4 && cr == 2 ? get_cell<PREC, C>(w[i], 1, 1.0f) : before;
+        }
+        if constexpr (HET) {
+          inner_ph = __shfl_up_sync(kFull, ph[C - 1], 1);
+          inner_k = __shfl_up_sync(kFull, k[C - 1], 1);
+          if (C == 4 && cr == 2) {
+            inner_ph = ph[1];
+            inner_k = k[1];
+          }
+        }
+        patch_cell(-1, y, e, eg, inner, unused);
+      }
+    }
 #pragma unroll
       for (int h = 0; h < C / 2; ++h) {
         const int ca = 2 * h, cb = ca + 1;
@@ -272,13 +295,20 @@ struct RowOps {
         }
         patch_cell(ca, y, e, eg, da, ga);
         patch_cell(cb, y, e, eg, db, gb);
-        PairMedium m;
+        Coef ma, mb;
         if constexpr (HET) {
           const float* sv = P.sv ? P.sv + (int64_t)y * P.pitch : nullptr;
-          m = pair_medium(coef_of(P, ph[ca], k[ca], sv ? __ldg(sv + col(ca)) : P.s_v), coef_of(P, ph[cb], k[cb], sv ? __ldg(sv + col(cb)) : P.s_v));
+          ma = coef_of(P, ph[ca], k[ca], sv ? __ldg(sv + col(ca)) : P.s_v);
+          mb = coef_of(P, ph[cb], k[cb], sv ? __ldg(sv + col(cb)) : P.s_v);
         } else {
-          m = pair_medium(coef_uniform(P), coef_uniform(P));
+          ma = mb = coef_uniform(P);
         }
+        if constexpr (kPressure) {
+          if (inlet && h == 0) pressure_cell(P, db, mb, ma, P.p_in, da);
+          if (outlet && cr == ca) pressure_cell(P, inner, HET ? coef_of(P, inner_ph, inner_k, P.s_v) : ma, ma, P.p_out, da);
+          if (outlet && cr == cb) pressure_cell(P, da, ma, mb, P.p_out, db);
+        }
+        const PairMedium m = pair_medium(ma, mb);
         float2 d[8], g[5], n0, ay = f2(P.ay), ux, uy;
 #pragma unroll
         for (int i = 0; i < 8; ++i) d[i] = make_float2(da[i], db[i]);

@@ -289,6 +289,8 @@ __device__ __forceinline__ void step_item(const StepParams& P, const Tiling& tl,
 // at 96), 5 (96) for the scalar 16-bit temperature step of a per-cell medium.
 template <int PREC, bool HET, bool THERMAL>
 __global__ void __launch_bounds__(kStepThreads, THERMAL ? (PREC != PREC_FP32 && HET ? 5 : 6) : 8) k_step(const StepParams P, Tiling tl) {
+  launch_dependents();
+  wait_prerequisites();
   step_item<PREC, HET, THERMAL, kStepThreads>(P, tl, blockIdx.x);
 }
 
@@ -296,6 +298,9 @@ template <int PREC, bool HET, bool THERMAL>
 static cudaError_t launch_step_t(const StepParams& P, cudaStream_t s) {
   const Tiling tl = tiling_of(P.nx, P.ny, P.bc_y, kStepThreads, true);
   const long long blocks = (long long)tl.frame_blocks + main_items(tl, P.ny, kStepThreads);
+  // launched early where the lattice fills the chip (1024^2 FP16 7.5 -> 7.25 us per step); a smaller
+  // launch would spread unevenly over the SMs that the one before still uses (640^2 5.6 -> 6.4)
+  if (blocks >= 8 * sm_count()) return launch_early(k_step<PREC, HET, THERMAL>, dim3((unsigned)blocks), dim3(kStepThreads), 0, s, P, tl);
   k_step<PREC, HET, THERMAL><<<(unsigned)blocks, kStepThreads, 0, s>>>(P, tl);
   return cudaGetLastError();
 }
@@ -358,9 +363,11 @@ __global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 1024 : 768) / NT) k_s
 // (512-lattice ensemble): FP16 at 72 registers 122.1 GLUPS (117.7 at 64, 112.9 at 80; the staged
 // form 102.4), BF16 and FP32 at 64 (BF16 113.4-114.7 at 64-80).
 template <int PREC, int NT>
-__global__ void __launch_bounds__(NT, (PREC == PREC_FP16 ? 896 : 1024) / NT)
+__global__ void __launch_bounds__(NT, (PREC == PREC_BF16 ? 1024 : 896) / NT)
     k_step_batch_items_shared(const StepParams U, const BatchRec* __restrict__ R, const StepParams* __restrict__ Pd,
                               const int64_t* __restrict__ item_start, const int* __restrict__ item_lattice, int flat) {
+  launch_dependents();
+  wait_prerequisites();
   const int d = item_lattice[blockIdx.x];
   const BatchRec& r = R[d];
   const Tiling tl = tiling_of(r.nx, r.ny, r.bc_y, NT, flat != 0);
@@ -460,21 +467,20 @@ static cudaError_t launch_batch_p(const StepParams* Pd, const int64_t* item_star
 }
 
 template <int PREC>
-static void launch_shared_p(const StepParams& U, const BatchRec* R, const StepParams* Pd, const int64_t* item_start,
+static cudaError_t launch_shared_p(const StepParams& U, const BatchRec* R, const StepParams* Pd, const int64_t* item_start,
                             const int* item_lattice, int64_t total, int nt, int flat, cudaStream_t s) {
   switch (nt) {
-    case 64: k_step_batch_items_shared<PREC, 64><<<(unsigned)total, 64, 0, s>>>(U, R, Pd, item_start, item_lattice, flat); break;
-    case 256: k_step_batch_items_shared<PREC, 256><<<(unsigned)total, 256, 0, s>>>(U, R, Pd, item_start, item_lattice, flat); break;
-    default: k_step_batch_items_shared<PREC, 128><<<(unsigned)total, 128, 0, s>>>(U, R, Pd, item_start, item_lattice, flat); break;
+    case 64: return launch_early(k_step_batch_items_shared<PREC, 64>, dim3((unsigned)total), dim3(64), 0, s, U, R, Pd, item_start, item_lattice, flat);
+    case 256: return launch_early(k_step_batch_items_shared<PREC, 256>, dim3((unsigned)total), dim3(256), 0, s, U, R, Pd, item_start, item_lattice, flat);
+    default: return launch_early(k_step_batch_items_shared<PREC, 128>, dim3((unsigned)total), dim3(128), 0, s, U, R, Pd, item_start, item_lattice, flat);
   }
 }
 
 cudaError_t launch_step_batch_shared(const StepParams& U, const BatchRec* R, const StepParams* Pd, const int64_t* item_start,
                                      const int* item_lattice, int64_t total, int prec, int nt, int flat, cudaStream_t s) {
-  if (prec == PREC_FP16) launch_shared_p<PREC_FP16>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
-  else if (prec == PREC_BF16) launch_shared_p<PREC_BF16>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
-  else launch_shared_p<PREC_FP32>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
-  return cudaGetLastError();
+  if (prec == PREC_FP16) return launch_shared_p<PREC_FP16>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
+  if (prec == PREC_BF16) return launch_shared_p<PREC_BF16>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
+  return launch_shared_p<PREC_FP32>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
 }
 
 // Largest number of CTAs of the persistent batched kernel (prec, nt) resident on one SM.

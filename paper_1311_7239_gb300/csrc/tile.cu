@@ -218,7 +218,8 @@ static size_t tile_bytes(int prec, bool het, bool thermal, int rows) {
 // saved), 512^2 4.9 / 3.6 / 5.3.  False where the lattice is left to the other kernels: above one wave,
 // and for the sides and widths that they treat differently (march_takes).
 static bool tile_shape(const StepParams& P, int prec, bool het, bool thermal, Tile& M) {
-  if (P.inplace || P.nx < 16 || P.ny < 16 || P.bc_x > BC_WALL || P.bc_y > BC_WALL) return false;
+  if (P.inplace || P.nx < 16 || P.ny < 16 || P.bc_x > BC_PRESSURE || P.bc_y > BC_WALL) return false;
+  if (P.bc_x == BC_PRESSURE && (prec != PREC_FP32 || thermal)) return false;
   if (P.bc_x == BC_PERIODIC && prec != PREC_FP32 && (P.nx & 3)) return false;
   if (het && thermal) return false;
   M.wrap = P.bc_x == BC_PERIODIC;
@@ -228,7 +229,10 @@ static bool tile_shape(const StepParams& P, int prec, bool het, bool thermal, Ti
   if (segs < 1) return false;
   if (segs > P.ny) segs = P.ny;
   M.height = (P.ny + segs - 1) / segs;
-  return tile_bytes(prec, het, thermal, M.height + 2 * M.halo) <= (size_t)kTileSmem;
+  // (16-bit storage, with its slower frame groups, falls behind single steps above 48 rows: 600^2 FP16
+  // with a per-cell medium 8.4 us per step against 7.2, 512^2 6.2 against 6.7)
+  const int rows = M.height + 2 * M.halo;
+  return tile_bytes(prec, het, thermal, rows) <= (size_t)kTileSmem && (prec == PREC_FP32 || rows <= 48);
 }
 
 int tile_steps(const StepParams& P, int prec, bool het, bool thermal) {
@@ -242,17 +246,7 @@ static cudaError_t launch_tile_t(const StepParams& P, const Tile& M, int prec, c
   auto fn = k_tile<PREC, HET, THERMAL>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c = {};
-  c.gridDim = dim3(M.strips * ((P.ny + M.height - 1) / M.height));
-  c.blockDim = dim3(kTileWarps * 32);
-  c.dynamicSmemBytes = bytes;
-  c.stream = s;
-  c.attrs = &at;
-  c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, fn, P, M);
+  return launch_early(fn, dim3(M.strips * ((P.ny + M.height - 1) / M.height)), dim3(kTileWarps * 32), bytes, s, P, M);
 }
 
 template <int PREC>
