@@ -228,7 +228,7 @@ LBM_API int lbm_residual_noalloc(const float* ux, const float* uy, const float* 
  * final state back into its own layout): runs the T steps -- the context ends at step T, as after lbm_step(ctx, T) -- and
  * returns the loss and its gradient with respect to the per-cell log K and eps (phi) fields,
  * including their effect on the initial equilibrium (Eq. 22).  Memory: checkpoints of the
- * post-collision state every ceil(sqrt(T)) steps, two segments of ceil(sqrt(T)) states (the
+ * post-collision state every ceil(sqrt(T)) steps, two segments of ceil(sqrt(T)) - 1 states (the
  * states of one segment are recomputed, on a second stream of lower priority, while the adjoint
  * steps of the next run on a stream of higher priority), two FP32 adjoint states and the gradient
  * sums (FP32 partial sums over at most 64 steps, folded into FP64 totals) form a workspace that

@@ -997,16 +997,16 @@ int lbm_adjoint(lbm_ctx* c, int T, int loss_kind, const float* target_ux, const 
   for (int k = 0; k < nck; ++k)
     if (!(ckpt[k] = ws_slot(c, 6 + k, fbytes, &rc, "cudaMalloc(checkpoints)"))) return rc;
   for (int h = 0; h < 2; ++h)
-    for (int j = 0; j < ck; ++j)
-      if (!(seg[h][j] = ws_slot(c, 6 + nck + h * ck + j, fbytes, &rc, "cudaMalloc(segment states)"))) return rc;
+    for (int j = 1; j < ck; ++j)  // (state 0 of a segment is its checkpoint)
+      if (!(seg[h][j] = ws_slot(c, 6 + nck + h * (ck - 1) + j - 1, fbytes, &rc, "cudaMalloc(segment states)"))) return rc;
   // In-place contexts: the sweep runs on two A-B state buffers of the workspace, from the same
   // initial state and with the same kernels as an A-B context; the final state is then written back
   // into the in-place layout (and the velocity of step T - 1 into the residual's record).
   const bool ip = c->inplace;
   void* ab[2] = {c->f[0], c->f[1]};
   for (int b = 0; ip && b < 2; ++b)
-    if (!(ab[b] = ws_slot(c, 6 + nck + 2 * ck + b, fbytes, &rc, "cudaMalloc(A-B states)"))) return rc;
-  ws_trim(c, 6 + nck + 2 * ck + (ip ? 2 : 0));
+    if (!(ab[b] = ws_slot(c, 6 + nck + 2 * (ck - 1) + b, fbytes, &rc, "cudaMalloc(A-B states)"))) return rc;
+  ws_trim(c, 6 + nck + 2 * (ck - 1) + (ip ? 2 : 0));
   if (ip && (rc = ensure_stage(c, 10 * n * sizeof(float)))) return rc;  // targets, then the final state
   StepParams B = params_for(c);
   B.inplace = 0;
@@ -1046,14 +1046,20 @@ int lbm_adjoint(lbm_ctx* c, int T, int loss_kind, const float* target_ux, const 
   LBM_CUDA(cudaMemsetAsync(hl, 0, hbytes, c->stream), "cudaMemset");
   LBM_CUDA(cudaMemsetAsync(hp, 0, hbytes, c->stream), "cudaMemset");
   const bool pressure = c->cfg.bc_x == LBM_PRESSURE;
-  // forward sweep, keeping the buffer before every ck-th step
-  for (int t = 0; t < T; ++t) {
+  // forward sweep, keeping the buffer before every ck-th step; in pairs of steps between those where the
+  // context takes them (the last step by itself: the state before it is kept, as by lbm_step)
+  const bool pairs = march_takes(ab_params(cur), c->prec, c->het, false);
+  for (int t = 0; t < T;) {
     if (t % ck == 0)
       LBM_CUDA(cudaMemcpyAsync(ckpt[t / ck], ab[cur], fbytes, cudaMemcpyDeviceToDevice, c->stream), "checkpoint copy");
-    LBM_CUDA(launch_step(ab_params(cur), c->prec, c->het, false, c->stream), "step kernel");
+    const int next = (t / ck + 1) * ck < T - 1 ? (t / ck + 1) * ck : T - 1;
+    const int k = pairs && t + 2 <= next ? 2 : 1;
+    LBM_CUDA(k == 2 ? launch_march(ab_params(cur), c->prec, c->het, false, c->stream)
+                    : launch_step(ab_params(cur), c->prec, c->het, false, c->stream), "step kernel");
     cur ^= 1;
-    ++c->steps;
-    ++c->history;
+    t += k;
+    c->steps += k;
+    c->history += k;
   }
   if (!ip) c->cur = cur;
   StepParams P = ab_params(cur);
@@ -1094,10 +1100,9 @@ int lbm_adjoint(lbm_ctx* c, int T, int loss_kind, const float* target_ux, const 
     const int t0 = k * ck, t1 = (t0 + ck < T) ? t0 + ck : T;
     std::vector<void*>& S = seg[k & 1];
     LBM_CUDA(cudaStreamWaitEvent(lo, freed[k & 1], 0), "cudaStreamWaitEvent");
-    LBM_CUDA(cudaMemcpyAsync(S[0], ckpt[k], fbytes, cudaMemcpyDeviceToDevice, lo), "checkpoint restore");
-    for (int j = 1; j < t1 - t0; ++j) {
+    for (int j = 1; j < t1 - t0; ++j) {  // (the segment's first state is the checkpoint)
       StepParams F = P;
-      F.src = S[j - 1];
+      F.src = j == 1 ? ckpt[k] : S[j - 1];
       F.dst = S[j];
       LBM_CUDA(launch_step(F, c->prec, c->het, false, lo), "recompute step");
     }
@@ -1112,7 +1117,7 @@ int lbm_adjoint(lbm_ctx* c, int T, int loss_kind, const float* target_ux, const 
       if (k > 0 && (rc2 = recompute(k - 1))) return rc2;
       LBM_CUDA(cudaStreamWaitEvent(hi, ready[k & 1], 0), "cudaStreamWaitEvent");
       for (int t = t1 - 1; t >= t0; --t) {
-        const void* buf = seg[k & 1][t - t0];
+        const void* buf = t == t0 ? ckpt[k] : seg[k & 1][t - t0];
         LBM_CUDA(launch_adj_step(P, c->prec, c->het, buf, nu[cur_nu], nu[cur_nu ^ 1], hl, hp, hi), "adjoint step");
         cur_nu ^= 1;
         if (walls) LBM_CUDA(launch_adj_wall(P, c->prec, c->het, buf, nu[cur_nu], hl, hp, hi), "adjoint wall nodes");
