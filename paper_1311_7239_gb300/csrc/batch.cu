@@ -67,6 +67,10 @@ struct lbm_batch {
   // fields that differ (one array per buffer parity) for the per-item kernel
   bool shared_consts = false;
   BatchRec* rec[2] = {nullptr, nullptr};
+  // A-B FP32 batches above the size of L2: work items of the kernels that take two steps per pass
+  MarchItem* pair_side = nullptr;
+  MarchItem* pair_main = nullptr;
+  int n_pair_side = 0, n_pair_main = 0;
   int cur = 0;
   int64_t steps = 0;
   int64_t cells = 0;
@@ -104,6 +108,8 @@ void release(lbm_batch* b) {
     cudaFree(b->dp[k]);
     cudaFree(b->rec[k]);
   }
+  cudaFree(b->pair_side);
+  cudaFree(b->pair_main);
   cudaFree(b->phi);
   cudaFree(b->K);
   cudaFree(b->walls);
@@ -191,11 +197,37 @@ int launch_once(lbm_batch* b, int cur, cudaStream_t s) {
   return LBM_OK;
 }
 
+cudaError_t launch_pair(const lbm_batch* b, int cur, cudaStream_t s) {
+  return launch_march_batch(b->dp[cur], b->pair_side, b->n_pair_side, b->pair_main, b->n_pair_main, s);
+}
+
+// Items of the pair kernels, if every lattice has a form that they handle and the batch is above the
+// size of L2 (march_takes).
+int set_pairs(lbm_batch* b) {
+  if (b->inplace || b->prec != PREC_FP32 || 2 * (uint64_t)b->pool_elems * b->elem < kMarchBytes) return LBM_OK;
+  std::vector<MarchItem> side, main;
+  for (int d = 0; d < b->n; ++d) {
+    if (!march_shape(b->hp[0][d], b->prec, true, false)) return LBM_OK;
+    march_items(b->hp[0][d], d, side, main);
+  }
+  int rc = balloc(b, reinterpret_cast<void**>(&b->pair_side), side.size() * sizeof(MarchItem), "cudaMalloc(pair items)");
+  if (rc == LBM_OK && !main.empty()) rc = balloc(b, reinterpret_cast<void**>(&b->pair_main), main.size() * sizeof(MarchItem), "cudaMalloc(pair items)");
+  if (rc) return rc;
+  LBM_BCUDA(cudaMemcpy(b->pair_side, side.data(), side.size() * sizeof(MarchItem), cudaMemcpyHostToDevice), "copy of the pair items");
+  if (!main.empty())
+    LBM_BCUDA(cudaMemcpy(b->pair_main, main.data(), main.size() * sizeof(MarchItem), cudaMemcpyHostToDevice), "copy of the pair items");
+  b->n_pair_side = (int)side.size();
+  b->n_pair_main = (int)main.size();
+  return LBM_OK;
+}
+
 int capture(lbm_batch* b, int cur) {
   if (!b->capture_stream) LBM_BCUDA(cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking), "cudaStreamCreate");
   LBM_BCUDA(cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
   cudaError_t le = cudaSuccess;
-  for (int k = 0; k < kBatchGraphSteps && le == cudaSuccess; ++k) le = launch_batch(b, cur ^ (k & 1), b->capture_stream);
+  const bool pairs = b->n_pair_side > 0;
+  for (int k = 0; k < (pairs ? kBatchGraphSteps / 2 : kBatchGraphSteps) && le == cudaSuccess; ++k)
+    le = pairs ? launch_pair(b, cur ^ (k & 1), b->capture_stream) : launch_batch(b, cur ^ (k & 1), b->capture_stream);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(b->capture_stream, &g);
   if (le != cudaSuccess || e != cudaSuccess) {
@@ -382,7 +414,7 @@ int lbm_batch_create(const lbm_config* cfgs, int n, lbm_batch** out) {
     }
     b->shared_consts = true;
   }
-  if ((rc = set_launch(b, b->inplace ? 128 : 64, 0)) || (rc = lbm_batch_init_equilibrium(b, -1, 1.0, 0.0, 0.0, 0))) {
+  if ((rc = set_pairs(b)) || (rc = set_launch(b, b->inplace ? 128 : 64, 0)) || (rc = lbm_batch_init_equilibrium(b, -1, 1.0, 0.0, 0.0, 0))) {
     release(b);
     return rc;
   }
@@ -458,6 +490,11 @@ int lbm_batch_step(lbm_batch* b, int n) {
     LBM_BCUDA(cudaGraphLaunch(b->graph[b->cur], b->stream), "cudaGraphLaunch");
     b->steps += kBatchGraphSteps;
     n -= kBatchGraphSteps;
+  }
+  for (; b->n_pair_side > 0 && n > 1; n -= 2) {
+    LBM_BCUDA(launch_pair(b, b->cur, b->stream), "batched step kernels");
+    b->cur ^= 1;
+    b->steps += 2;
   }
   for (int k = 0; k < n; ++k) {
     int rc = launch_once(b, b->cur, b->stream);

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -55,7 +57,15 @@ cudaError_t launch_step_batch(const StepParams* Pd, const int64_t* item_start, c
                               int nt, int grid, int flat, cudaStream_t s);
 cudaError_t launch_step(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);
 int sm_count();  // SMs of the current device
+constexpr uint64_t kMarchBytes = 100ull << 20;  // FP32 state (both buffers) from which steps are taken in pairs
+bool march_shape(const StepParams& P, int prec, bool het, bool thermal);
 bool march_takes(const StepParams& P, int prec, bool het, bool thermal);
+// A warp's work in the batched pair kernels: rows [ya, yb) (none if equal) of a strip of a lattice.
+struct MarchItem {
+  int lattice, strip, ya, yb, strips, wrap;
+};
+void march_items(const StepParams& P, int lattice, std::vector<MarchItem>& side, std::vector<MarchItem>& main);
+cudaError_t launch_march_batch(const StepParams* Pd, const MarchItem* side, int n_side, const MarchItem* main, int n_main, cudaStream_t s);
 int tile_steps(const StepParams& P, int prec, bool het, bool thermal);
 cudaError_t launch_tile(const StepParams& P, int prec, bool het, bool thermal, int steps, cudaStream_t s);
 cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);

@@ -392,14 +392,18 @@ __global__ void __launch_bounds__(kMarchThreads, CTAS) k_march(const __grid_cons
 // temperature 40.8 -> 45.5).
 bool march_takes(const StepParams& P, int prec, bool het, bool thermal) {
   const uint64_t bytes = 2 * (uint64_t)(thermal ? 13 : 8) * (uint64_t)P.nx * P.ny * (prec == PREC_FP32 ? 4 : 2);
-  if (bytes < (prec == PREC_FP32 ? 100ull << 20 : 120ull << 20)) return false;
+  if (bytes < (prec == PREC_FP32 ? kMarchBytes : 120ull << 20)) return false;
   if (prec != PREC_FP32 && (het || thermal)) return false;
+  return march_shape(P, prec, het, thermal);
+}
+
+// The sides and sizes that the pair kernels handle.
+bool march_shape(const StepParams& P, int prec, bool het, bool thermal) {
   if (P.inplace || P.nx < 16 || P.ny < 16) return false;
   if (P.bc_x > BC_PRESSURE || P.bc_y > BC_WALL || (P.bc_x == BC_PRESSURE && (prec != PREC_FP32 || thermal))) return false;
   if (P.bc_x == BC_PERIODIC && prec != PREC_FP32 && (P.nx & 3)) return false;
   if (het && thermal) return false;
-  if (8 * (uint64_t)P.plane * (prec == PREC_FP32 ? 4 : 2) / 16 >= (1ull << 32)) return false;  // (fill's 32-bit offsets)
-  return true;
+  return 8 * (uint64_t)P.plane * (prec == PREC_FP32 ? 4 : 2) / 16 < (1ull << 32);  // (fill's 32-bit offsets)
 }
 
 int sm_count() {
@@ -466,6 +470,76 @@ cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, 
     case PREC_FP16: return launch_march_p<PREC_FP16>(P, het, thermal, s);
     default: return launch_march_p<PREC_BF16>(P, het, thermal, s);
   }
+}
+
+// --------------------------------------------------------------------------------------------
+// Batched ensembles (FP32, per-cell media): the same pairs of steps for all lattices of a batch in one
+// launch of each kernel.  A CTA's four warps take four items of one lattice, whose parameters are
+// staged in shared memory; the items of a lattice are padded to whole CTAs.
+// --------------------------------------------------------------------------------------------
+constexpr int kBatchC = 2, kBatchStages = 3;
+
+template <bool SIDE>
+__global__ void __launch_bounds__(kMarchThreads, SIDE ? 1 : 4)
+    k_march_batch(const StepParams* __restrict__ Pd, const MarchItem* __restrict__ items) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ StepParams sP;
+  using Inner = Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, false, false>;
+  if (SIDE) launch_dependents();
+  const MarchItem it = items[blockIdx.x * (kMarchThreads / 32) + (threadIdx.x >> 5)];
+  static_assert(sizeof(StepParams) % 8 == 0, "parameters are copied as 8-byte words");
+  const unsigned long long* from = reinterpret_cast<const unsigned long long*>(Pd + it.lattice);
+  for (int i = threadIdx.x; i < (int)(sizeof(StepParams) / 8); i += kMarchThreads) reinterpret_cast<unsigned long long*>(&sP)[i] = from[i];
+  __syncthreads();
+  char* buf = smem + (threadIdx.x >> 5) * (kBatchStages * Inner::kStage);
+  March M;
+  M.strips = it.strips;
+  M.wrap = it.wrap;
+  if (it.ya < it.yb) {
+    if constexpr (!SIDE) {
+      Inner m(sP, buf);
+      m.run(M, it.strip, it.ya, it.yb);
+    } else if (it.ya == 0 || it.yb == sP.ny) {
+      Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, true, true> m(sP, buf);
+      m.run(M, it.strip, it.ya, it.yb);
+    } else {
+      Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, true, false> m(sP, buf);
+      m.run(M, it.strip, it.ya, it.yb);
+    }
+  }
+  if (!SIDE) wait_prerequisites();
+}
+
+// Items of one lattice, in whole CTAs (kMarchThreads / 32 items).
+void march_items(const StepParams& P, int lattice, std::vector<MarchItem>& side, std::vector<MarchItem>& main) {
+  const bool wrap = P.bc_x == BC_PERIODIC;
+  const int strips = march_strips<PREC_FP32, kBatchC>(P.nx, wrap), ny = P.ny, rows = 24, side_rows = 8;
+  auto pad = [&](std::vector<MarchItem>& v) {
+    while (v.size() % (kMarchThreads / 32)) v.push_back(MarchItem{lattice, 0, 0, 0, strips, wrap});
+  };
+  for (int k = 0; k < strips; ++k) {
+    const int x = march_x0<PREC_FP32, kBatchC>(k, wrap);
+    const bool inner = x >= 4 && x + 32 * kBatchC <= (P.nx - 1) / 4 * 4;
+    side.push_back(MarchItem{lattice, k, 0, kMarchSide, strips, wrap});
+    side.push_back(MarchItem{lattice, k, ny - kMarchSide, ny, strips, wrap});
+    const int step = inner ? rows : side_rows;
+    for (int y = kMarchSide; y < ny - kMarchSide; y += step)
+      (inner ? main : side).push_back(MarchItem{lattice, k, y, y + step < ny - kMarchSide ? y + step : ny - kMarchSide, strips, wrap});
+  }
+  pad(side);
+  pad(main);
+}
+
+cudaError_t launch_march_batch(const StepParams* Pd, const MarchItem* side, int n_side, const MarchItem* main, int n_main, cudaStream_t s) {
+  const size_t bytes = (kMarchThreads / 32) * kBatchStages * Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, false, false>::kStage;
+  auto sides = k_march_batch<true>;
+  auto inner = k_march_batch<false>;
+  cudaError_t e = cudaFuncSetAttribute(sides, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(inner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  sides<<<n_side / 4, kMarchThreads, bytes, s>>>(Pd, side);
+  if ((e = cudaGetLastError()) != cudaSuccess || n_main == 0) return e;
+  return launch_early(inner, dim3(n_main / 4), dim3(kMarchThreads), bytes, s, Pd, main);
 }
 
 }  // namespace lbm
