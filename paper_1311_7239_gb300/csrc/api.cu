@@ -139,8 +139,8 @@ struct lbm_ctx {
   float* phi = nullptr;
   float* K = nullptr;
   float* sv = nullptr;  // per-cell viscous rate (heterogeneous mode), when a viscosity-ratio field is set
-  std::vector<void*> ws;       // adjoint workspace, kept between lbm_adjoint calls (slots, see lbm_adjoint)
-  std::vector<size_t> ws_bytes;
+  char* ws = nullptr;          // adjoint workspace, kept between lbm_adjoint calls (cut into buffers there)
+  size_t ws_bytes = 0;
   bool het = false;
   unsigned int* err = nullptr;   // device error word
   float* walls = nullptr;        // wall velocities [4][2] read by the kernels
@@ -395,7 +395,7 @@ void release(lbm_ctx* c) {
   cudaFree(c->probe);
   cudaFree(c->red);
   cudaFree(c->stage);
-  for (void* p : c->ws) cudaFree(p);
+  cudaFree(c->ws);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -901,40 +901,23 @@ int lbm_nusselt(lbm_ctx* c, int side, double* nu) {
 
 namespace {
 
-// Device buffers of one adjoint run, freed on every exit path.
-// Slot k of the adjoint workspace, `bytes` long: the buffer kept from an earlier call when its
-// size matches, else a new allocation.  Callers synchronise before the workspace changes hands.
-void* ws_slot(lbm_ctx* c, size_t k, size_t bytes, int* rc, const char* what) {
-  if (c->ws.size() <= k) {
-    c->ws.resize(k + 1, nullptr);
-    c->ws_bytes.resize(k + 1, 0);
-  }
-  if (c->ws[k] && c->ws_bytes[k] == bytes) return c->ws[k];
-  if (c->ws[k]) {
-    cudaFree(c->ws[k]);
-    c->bytes -= c->ws_bytes[k];
-    c->ws[k] = nullptr;
-    c->ws_bytes[k] = 0;
-  }
-  void* p = nullptr;
-  if ((*rc = dev_alloc(c, &p, bytes, what)) != LBM_OK) return nullptr;
-  c->ws[k] = p;
-  c->ws_bytes[k] = bytes;
-  return p;
+void ws_release(lbm_ctx* c) {
+  if (!c->ws) return;
+  cudaFree(c->ws);
+  c->bytes -= c->ws_bytes;
+  c->ws = nullptr;
+  c->ws_bytes = 0;
 }
 
-// Frees the workspace slots from `keep` on.
-void ws_trim(lbm_ctx* c, size_t keep) {
-  for (size_t k = keep; k < c->ws.size(); ++k) {
-    if (c->ws[k]) {
-      cudaFree(c->ws[k]);
-      c->bytes -= c->ws_bytes[k];
-    }
-  }
-  if (c->ws.size() > keep) {
-    c->ws.resize(keep);
-    c->ws_bytes.resize(keep);
-  }
+// The adjoint workspace, `bytes` long: the one kept from an earlier call when its size matches, else a
+// new one.  A single allocation: one per buffer took 3.7 ms of a 16 ms gradient (T = 100, 2048 x 1024)
+// to make and free.  Callers synchronise before the workspace changes hands.
+int ws_reserve(lbm_ctx* c, size_t bytes) {
+  if (c->ws && c->ws_bytes == bytes) return LBM_OK;
+  ws_release(c);
+  const int rc = dev_alloc(c, reinterpret_cast<void**>(&c->ws), bytes, "cudaMalloc(adjoint workspace)");
+  if (rc == LBM_OK) c->ws_bytes = bytes;
+  return rc;
 }
 
 int copy_out(lbm_ctx* c, void* user, const void* dev, size_t bytes, bool* waited) {
@@ -977,36 +960,39 @@ int lbm_adjoint(lbm_ctx* c, int T, int loss_kind, const float* target_ux, const 
   int ck = 1;
   while ((int64_t)ck * ck < T) ++ck;  // checkpoint interval ceil(sqrt(T))
   const int nck = (T + ck - 1) / ck;
-  // workspace slots (kept between calls): 0-1 adjoint state, 2-3 FP64 gradient totals, 4-5 FP32
-  // gradient partial sums, then nck checkpoints and two sets of ck segment states
-  LBM_CUDA(cudaStreamSynchronize(c->stream), "stream synchronize");
-  int rc = LBM_OK;
-  float* nu[2];
-  for (int b = 0; b < 2; ++b)
-    if (!(nu[b] = static_cast<float*>(ws_slot(c, b, nubytes, &rc, "cudaMalloc(adjoint state)")))) return rc;
-  const size_t gbytes = (size_t)c->plane * sizeof(double);  // pitched [ny][pitch]
-  const size_t hbytes = (size_t)c->plane * sizeof(float);
-  double* gl = static_cast<double*>(ws_slot(c, 2, gbytes, &rc, "cudaMalloc(gradients)"));
-  double* gp = gl ? static_cast<double*>(ws_slot(c, 3, gbytes, &rc, "cudaMalloc(gradients)")) : nullptr;
-  float* hl = gp ? static_cast<float*>(ws_slot(c, 4, hbytes, &rc, "cudaMalloc(gradient partial sums)")) : nullptr;
-  float* hp = hl ? static_cast<float*>(ws_slot(c, 5, hbytes, &rc, "cudaMalloc(gradient partial sums)")) : nullptr;
-  if (!hp) return rc;
-  // two sets of segment states: the adjoint steps of one segment read one set while the states of
-  // the segment before it are recomputed into the other
-  std::vector<void*> ckpt(nck), seg[2] = {std::vector<void*>(ck), std::vector<void*>(ck)};
-  for (int k = 0; k < nck; ++k)
-    if (!(ckpt[k] = ws_slot(c, 6 + k, fbytes, &rc, "cudaMalloc(checkpoints)"))) return rc;
-  for (int h = 0; h < 2; ++h)
-    for (int j = 1; j < ck; ++j)  // (state 0 of a segment is its checkpoint)
-      if (!(seg[h][j] = ws_slot(c, 6 + nck + h * (ck - 1) + j - 1, fbytes, &rc, "cudaMalloc(segment states)"))) return rc;
   // In-place contexts: the sweep runs on two A-B state buffers of the workspace, from the same
   // initial state and with the same kernels as an A-B context; the final state is then written back
   // into the in-place layout (and the velocity of step T - 1 into the residual's record).
   const bool ip = c->inplace;
+  LBM_CUDA(cudaStreamSynchronize(c->stream), "stream synchronize");
+  // the workspace: two adjoint states, FP64 gradient totals, FP32 gradient partial sums, nck
+  // checkpoints, two sets of ck - 1 segment states, in-place contexts' two states
+  const size_t gbytes = (size_t)c->plane * sizeof(double);  // pitched [ny][pitch]
+  const size_t hbytes = (size_t)c->plane * sizeof(float);
+  auto padded = [](size_t b) { return (b + 511) / 512 * 512; };
+  const size_t states = (size_t)nck + 2 * (size_t)(ck - 1) + (ip ? 2 : 0);
+  int rc = ws_reserve(c, 2 * (padded(nubytes) + padded(gbytes) + padded(hbytes)) + states * padded(fbytes));
+  if (rc) return rc;
+  char* at = c->ws;
+  auto take = [&](size_t b) {
+    void* p = at;
+    at += padded(b);
+    return p;
+  };
+  float* nu[2];
+  for (float*& p : nu) p = static_cast<float*>(take(nubytes));
+  double* gl = static_cast<double*>(take(gbytes));
+  double* gp = static_cast<double*>(take(gbytes));
+  float* hl = static_cast<float*>(take(hbytes));
+  float* hp = static_cast<float*>(take(hbytes));
+  // two sets of segment states: the adjoint steps of one segment read one set while the states of
+  // the segment before it are recomputed into the other (state 0 of a segment is its checkpoint)
+  std::vector<void*> ckpt(nck), seg[2] = {std::vector<void*>(ck), std::vector<void*>(ck)};
+  for (void*& p : ckpt) p = take(fbytes);
+  for (int h = 0; h < 2; ++h)
+    for (int j = 1; j < ck; ++j) seg[h][j] = take(fbytes);
   void* ab[2] = {c->f[0], c->f[1]};
-  for (int b = 0; ip && b < 2; ++b)
-    if (!(ab[b] = ws_slot(c, 6 + nck + 2 * (ck - 1) + b, fbytes, &rc, "cudaMalloc(A-B states)"))) return rc;
-  ws_trim(c, 6 + nck + 2 * (ck - 1) + (ip ? 2 : 0));
+  for (int b = 0; ip && b < 2; ++b) ab[b] = take(fbytes);
   if (ip && (rc = ensure_stage(c, 10 * n * sizeof(float)))) return rc;  // targets, then the final state
   StepParams B = params_for(c);
   B.inplace = 0;
@@ -1157,7 +1143,7 @@ int lbm_adjoint_step(lbm_ctx* c, int T, int loss_kind, const float* target_ux, c
 int lbm_release_workspace(lbm_ctx* c) {
   if (!c) return fail(LBM_EINVAL, "null context");
   LBM_CUDA(cudaStreamSynchronize(c->stream), "stream synchronize");
-  ws_trim(c, 0);
+  ws_release(c);
   return LBM_OK;
 }
 
