@@ -32,6 +32,16 @@ PREC = {"fp32": 0, "fp16": 1, "bf16": 2}
 BYTES_PER_LU = {"fp32": 64, "fp16": 32, "bf16": 32}
 
 
+def steps_per_pass(prec, cells, populations=8, plain=True, sides="halfway"):
+    """Time steps that one pass over the populations takes (A-B streaming): two where the state is larger
+    than L2 (plain: no per-cell medium and no temperature), so that an update moves half the bytes."""
+    state = 2 * populations * cells * (4 if prec == "fp32" else 2)
+    if sides != "halfway":
+        return 1
+    return 2 if state >= (100 << 20 if prec == "fp32" else 120 << 20) and (plain or prec == "fp32") else 1
+
+
+
 def max_over_ranks(value, dist, device):
     """The largest of the ranks' values (the slowest rank's time), on every rank."""
     import torch
@@ -353,6 +363,7 @@ def thermal_form(lbm, L, steps, warmup, local_rank):
         lat.sync()
         lat.close()
         ms = start.elapsed_time(stop)
+        bpl /= steps_per_pass(prec, L * L, 13, plain=False)
         bw = bpl * L * L * steps / (ms * 1e-3) / 1e9
         out[prec] = {"value": L * L * steps / (ms * 1e-3) / 1e6, "unit": "MLUPS", "achieved_gbs": bw, "roofline_frac": bw / peak,
                      "algorithmic_bytes_per_lu": bpl, "steps": steps, "clocks": clk.summary()}
@@ -392,6 +403,7 @@ def heterogeneous_form(lbm, L, steps, warmup, local_rank):
         lat.sync()
         lat.close()
         ms = start.elapsed_time(stop)
+        bpl /= steps_per_pass(prec, L * L, plain=False)
         bw = bpl * L * L * steps / (ms * 1e-3) / 1e9
         out[name] = {"value": L * L * steps / (ms * 1e-3) / 1e6, "unit": "MLUPS", "achieved_gbs": bw, "roofline_frac": bw / peak,
                      "algorithmic_bytes_per_lu": bpl, "steps": steps, "clocks": clk.summary()}
@@ -438,6 +450,8 @@ def ensemble_form(lbm, steps, local_rank):
         b.sync()
         b.close()
         bpl = BYTES_PER_LU[prec] + 8  # + per-cell eps and K
+        if key == "fp32":
+            bpl /= steps_per_pass(prec, cells, plain=False)
         mlups = cells * steps / (ms_b * 1e-3) / 1e6
         res[key] = {"batched_MLUPS": mlups, "one_by_one_MLUPS": cells * each / (ms_e * 1e-3) / 1e6,
                     "batched_roofline_frac": mlups * 1e6 * bpl / 1e9 / peak, "algorithmic_bytes_per_lu": bpl,
@@ -591,13 +605,15 @@ def run_gpu(args, rank, world, local_rank):
                 continue
             ms_o, clk_o, lat_o = timed_steps(lbm, L, other, max(3, args.steps // 2), args.warmup, local_rank, dist)
             lat_o.close()
-            bw = BYTES_PER_LU[other] * cells / (ms_o * 1e-3 / max(3, args.steps // 2)) / 1e9
+            bpl_o = BYTES_PER_LU[other] / (1 if streaming else steps_per_pass(other, cells, sides=args.walls))
+            bw = bpl_o * cells / (ms_o * 1e-3 / max(3, args.steps // 2)) / 1e9
             forms[other] = {"value": cells * max(3, args.steps // 2) / (ms_o * 1e-3) / 1e6, "unit": "MLUPS",
-                            "roofline_frac": bw / peak, "achieved_gbs": bw, "algorithmic_bytes_per_lu": BYTES_PER_LU[other],
+                            "roofline_frac": bw / peak, "achieved_gbs": bw, "algorithmic_bytes_per_lu": bpl_o,
                             "clocks": clk_o}
     if rank != 0:
         return 0
-    bpl = BYTES_PER_LU[prec]
+    per_pass = 1 if streaming else steps_per_pass(prec, cells, sides=args.walls)
+    bpl = BYTES_PER_LU[prec] / per_pass
     achieved = bpl * cells / (ms * 1e-3 / args.steps) / 1e9
     kernel_key = (f"k_step_{prec}_uniform_{L}" if not streaming else f"k_step_ip_{prec}_uniform_{L}") + ("_nee" if args.walls == "nee" else "")
     traffic = traffic_for(kernel_key)
@@ -609,10 +625,10 @@ def run_gpu(args, rank, world, local_rank):
                                f"{prec} deviation storage, {'in-place' if streaming else 'A-B pull'} streaming"
                                + (", extrapolated wall nodes" if args.walls == "nee" else ""),
                    "nx": L, "ny": L, "precision": prec,
-                   "l2": f"inputs larger than L2 ({1 if streaming else 2} population buffer(s) of {bpl // 2 * cells / 1e6:.0f} MB)",
+                   "l2": f"inputs larger than L2 ({1 if streaming else 2} population buffer(s) of {BYTES_PER_LU[prec] // 2 * cells / 1e6:.0f} MB)",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": traffic, "peak_source": f"{peak_kind} hbm_gbs", "kernel": "k_step_ip" if streaming else "k_step",
+                     "traffic": traffic, "peak_source": f"{peak_kind} hbm_gbs", "kernel": "k_step_ip" if streaming else "k_march" if per_pass == 2 else "k_step",
                      "algorithmic_bytes_per_lu": bpl},
         "gpu_launches": args.steps,
         "e2e": {"value": e2e_mlups, "unit": "MLUPS", "h2d_bytes_per_step": int(walls.numel() * 4),
@@ -715,7 +731,8 @@ def run_sweep(args, local_rank):
                                        streaming=1 if args.streaming == "inplace" else 0, walls=args.walls)
             lat.close()
             cells = L * L
-            bw = BYTES_PER_LU[prec] * cells * steps / (ms * 1e-3) / 1e9
+            per_pass = 1 if args.streaming == "inplace" else steps_per_pass(prec, cells, sides=args.walls)
+            bw = BYTES_PER_LU[prec] / per_pass * cells * steps / (ms * 1e-3) / 1e9
             l2 = 2 * BYTES_PER_LU[prec] // 2 * cells / 1e6
             print(json.dumps({"size": L, "precision": prec, "streaming": args.streaming, "steps": steps,
                               "MLUPS": cells * steps / (ms * 1e-3) / 1e6,

@@ -202,8 +202,11 @@ cudaError_t launch_pair(const lbm_batch* b, int cur, cudaStream_t s) {
 }
 
 // Items of the pair kernels, if every lattice has a form that they handle and the batch is above the
-// size of L2 (march_takes).
+// size of L2 (march_takes).  Small lattices are mostly sides, whose warps are slower: GLUPS of single
+// steps -> pairs 68 -> 48 at 24 thousand cells per lattice on average, 75 -> 76 at 94, 81 -> 92 at 165,
+// 84 -> 104 at 288, 84 -> 113 at 920.
 int set_pairs(lbm_batch* b) {
+  if (b->cells < 120000 * (int64_t)b->n) return LBM_OK;
   if (b->inplace || b->prec != PREC_FP32 || 2 * (uint64_t)b->pool_elems * b->elem < kMarchBytes) return LBM_OK;
   std::vector<MarchItem> side, main;
   for (int d = 0; d < b->n; ++d) {
