@@ -435,15 +435,23 @@ static cudaError_t launch_ip_t(const StepParams& P, cudaStream_t s) {
   const int groups = (P.nx + kIpCells - 1) / kIpCells;
   const int gx = (groups + kIpThreads - 1) / kIpThreads;
   const long long blocks = (long long)frame_blocks + (long long)gx * P.ny;
+  const bool early = blocks >= 8 * sm_count();  // launched early where the lattice fills the chip (as k_step)
   if (P.edge) {  // the boundary nodes' states, before the step overwrites their neighbours' slots
     const int64_t threads = 8 * 2 * ((int64_t)P.nx + P.ny);
-    const cudaError_t e = launch_early(k_edge_ip<PREC, HET, THERMAL>, dim3((unsigned)((threads + 127) / 128)), dim3(128), 0, s, P);
-    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((threads + 127) / 128));
+    if (early) {
+      const cudaError_t e = launch_early(k_edge_ip<PREC, HET, THERMAL>, grid, dim3(128), 0, s, P);
+      if (e != cudaSuccess) return e;
+    } else {
+      k_edge_ip<PREC, HET, THERMAL><<<grid, 128, 0, s>>>(P);
+    }
   }
   // the variant that records u runs once per lbm_step call
   auto fn = P.urec ? (P.parity ? k_step_ip<PREC, HET, THERMAL, 1, true> : k_step_ip<PREC, HET, THERMAL, 0, true>)
                    : (P.parity ? k_step_ip<PREC, HET, THERMAL, 1, false> : k_step_ip<PREC, HET, THERMAL, 0, false>);
-  return launch_early(fn, dim3((unsigned)blocks), dim3(kIpThreads), 0, s, P, frame_blocks, gx);
+  if (early) return launch_early(fn, dim3((unsigned)blocks), dim3(kIpThreads), 0, s, P, frame_blocks, gx);
+  fn<<<(unsigned)blocks, kIpThreads, 0, s>>>(P, frame_blocks, gx);
+  return cudaGetLastError();
 }
 
 template <int PREC>
