@@ -155,7 +155,7 @@ struct lbm_ctx {
   // parameters of the last lbm_init_equilibrium (the initial state the adjoint differentiates)
   double init_p0 = 1.0, init_ux = 0.0, init_uy = 0.0;
   int init_phip = 0;
-  // CUDA graphs of kGraphSteps steps starting from buffer 0 or 1 (captured on first use)
+  // CUDA graphs of several steps (Pace::graph) starting from buffer 0 or 1 (captured on first use)
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaStream_t capture_stream = nullptr;
   // adjoint reverse sweep: the adjoint steps on a high-priority stream, the recomputation of the

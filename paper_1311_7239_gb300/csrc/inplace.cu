@@ -69,8 +69,6 @@ __device__ __forceinline__ bool boundary_node(const StepParams& P, int x, int y)
 // stores its own population.
 template <int PREC, bool HET, bool THERMAL>
 __global__ void k_edge_ip(const StepParams P) {
-  launch_dependents();
-  wait_prerequisites();
   using T = typename Store<PREC>::T;
   const int n = 2 * (P.nx + P.ny);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -402,8 +400,6 @@ __device__ __forceinline__ void ip_block(const StepParams& P, int frame_blocks, 
 // temperature populations (96; at 80 the FP32 thermal step spills).
 template <int PREC, bool HET, bool THERMAL, int PAR, bool REC>
 __global__ void __launch_bounds__(kIpThreads, THERMAL ? 5 : (PREC == PREC_FP32 ? 8 : 7)) k_step_ip(const StepParams P, int frame_blocks, int gx) {
-  launch_dependents();
-  wait_prerequisites();
   ip_block<PREC, HET, THERMAL, PAR, REC>(P, frame_blocks, gx, (int)blockIdx.x);
 }
 
@@ -435,22 +431,21 @@ static cudaError_t launch_ip_t(const StepParams& P, cudaStream_t s) {
   const int groups = (P.nx + kIpCells - 1) / kIpCells;
   const int gx = (groups + kIpThreads - 1) / kIpThreads;
   const long long blocks = (long long)frame_blocks + (long long)gx * P.ny;
-  const bool early = blocks >= 8 * sm_count();  // launched early where the lattice fills the chip (as k_step)
   if (P.edge) {  // the boundary nodes' states, before the step overwrites their neighbours' slots
     const int64_t threads = 8 * 2 * ((int64_t)P.nx + P.ny);
-    const dim3 grid((unsigned)((threads + 127) / 128));
-    if (early) {
-      const cudaError_t e = launch_early(k_edge_ip<PREC, HET, THERMAL>, grid, dim3(128), 0, s, P);
-      if (e != cudaSuccess) return e;
-    } else {
-      k_edge_ip<PREC, HET, THERMAL><<<grid, 128, 0, s>>>(P);
-    }
+    k_edge_ip<PREC, HET, THERMAL><<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(P);
   }
   // the variant that records u runs once per lbm_step call
-  auto fn = P.urec ? (P.parity ? k_step_ip<PREC, HET, THERMAL, 1, true> : k_step_ip<PREC, HET, THERMAL, 0, true>)
-                   : (P.parity ? k_step_ip<PREC, HET, THERMAL, 1, false> : k_step_ip<PREC, HET, THERMAL, 0, false>);
-  if (early) return launch_early(fn, dim3((unsigned)blocks), dim3(kIpThreads), 0, s, P, frame_blocks, gx);
-  fn<<<(unsigned)blocks, kIpThreads, 0, s>>>(P, frame_blocks, gx);
+  if (P.urec) {
+    if (P.parity)
+      k_step_ip<PREC, HET, THERMAL, 1, true><<<(unsigned)blocks, kIpThreads, 0, s>>>(P, frame_blocks, gx);
+    else
+      k_step_ip<PREC, HET, THERMAL, 0, true><<<(unsigned)blocks, kIpThreads, 0, s>>>(P, frame_blocks, gx);
+  } else if (P.parity) {
+    k_step_ip<PREC, HET, THERMAL, 1, false><<<(unsigned)blocks, kIpThreads, 0, s>>>(P, frame_blocks, gx);
+  } else {
+    k_step_ip<PREC, HET, THERMAL, 0, false><<<(unsigned)blocks, kIpThreads, 0, s>>>(P, frame_blocks, gx);
+  }
   return cudaGetLastError();
 }
 

@@ -361,7 +361,8 @@ __global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 1024 : 768) / NT) k_s
 // staging the parameter set in shared memory and keeps the constants out of the registers.  Frame
 // items, which use every parameter, stage the lattice's set as the general form.  Register caps
 // (512-lattice ensemble): FP16 at 72 registers 122.1 GLUPS (117.7 at 64, 112.9 at 80; the staged
-// form 102.4), BF16 and FP32 at 64 (BF16 113.4-114.7 at 64-80).
+// form 102.4), BF16 at 64 (113.4-114.7 at 64-80), FP32 at 72 (48 lattices 85.3 GLUPS, 81.7 at 64, which
+// its collision with written-out roundings spills).
 template <int PREC, int NT>
 __global__ void __launch_bounds__(NT, (PREC == PREC_BF16 ? 1024 : 896) / NT)
     k_step_batch_items_shared(const StepParams U, const BatchRec* __restrict__ R, const StepParams* __restrict__ Pd,
