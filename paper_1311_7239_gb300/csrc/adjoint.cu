@@ -275,8 +275,7 @@ __device__ __forceinline__ float group8_sum(float v, unsigned mask) {
 }
 
 template <int PREC, bool HET>
-__global__ void k_adj_nee(const StepParams P, const void* buf, float* __restrict__ nu, float* __restrict__ g_l,
-                          float* __restrict__ g_phi) {
+__global__ void k_adj_nee(const StepParams P, const void* buf, float* nu, float* g_l, float* g_phi) {
   launch_dependents();
   wait_prerequisites();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -403,7 +402,7 @@ __global__ void k_adj_wall(const StepParams P, const void* buf, WallGroups G, fl
     const float lam = nu[i * P.plane + ob];
     nu[i * P.plane + ob] = 0.0f;
     const Coef cb = coef_at<HET>(P, bx[k], by[k]);
-    const float uwx = __ldg(P.uw + 2 * bw[k]), uwy = __ldg(P.uw + 2 * bw[k] + 1);
+    const float uwx = wall_velocity(P, bw[k], 0), uwy = wall_velocity(P, bw[k], 1);
     const float euw = ex * uwx + ey * uwy;
     const float wl = wi * lam;
     const float W = group8_sum(wl, gm);

@@ -238,7 +238,7 @@ __global__ void k_macros(const StepParams P, float* __restrict__ p, float* __res
 
 // one cell's (p, ux, uy, T) into out[0..3] (T = 0 without a temperature field)
 template <int PREC, bool HET, bool THERMAL>
-__global__ void k_probe(const StepParams P, int x, int y, float* __restrict__ out) {
+__global__ void k_probe(const StepParams P, int x, int y, float* out) {
   launch_dependents();
   wait_prerequisites();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
@@ -280,9 +280,10 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
 
 // Pass 1: per-block partial sums of |u(t) - u(t-1)|^2 and |u(t)|^2 into partial[2 * block];
 // u(t-1) from the previous state (prev, gprev) or, if uprev is given, from its recorded
-// components (dense [2][ny][nx]).
+// components (dense [2][ny][nx]).  (Three CTAs per SM: left to itself the compiler interleaves the loads
+// of the walls of several cells, 72 -> 128 registers.)
 template <int PREC, bool HET, bool THERMAL>
-__global__ void k_residual_partial(const StepParams P, const void* prev, const void* gprev, const float* __restrict__ uprev,
+__global__ void __launch_bounds__(256, 3) k_residual_partial(const StepParams P, const void* prev, const void* gprev, const float* __restrict__ uprev,
                                    double* __restrict__ partial) {
   double num = 0.0, den = 0.0;
   const int64_t n = (int64_t)P.nx * P.ny;
@@ -438,7 +439,7 @@ cudaError_t launch_macros(const StepParams& P, int prec, bool het, bool thermal,
 }
 
 // a few floats, e.g. wall velocities from page-locked host memory that the device reads directly
-__global__ void k_copy_small(float* __restrict__ dst, const float* __restrict__ src, int n) {
+__global__ void k_copy_small(float* dst, const float* src, int n) {
   launch_dependents();
   wait_prerequisites();
   const int i = threadIdx.x;

@@ -738,14 +738,21 @@ __device__ __forceinline__ int64_t ip_source5(const StepParams& P, int x, int y,
   return ip_off5(P, sx, sy, opp5(i), P.parity);
 }
 
+// Component c of the velocity of wall w.  lbm_set_walls may write it while a kernel that was launched
+// early is already resident: an ordinary load that stays behind wait_prerequisites(), and not one
+// through the read-only path, which takes memory that is constant for as long as the kernel lives.
+// (A volatile one is as safe and slower where the frame's cells bound a step: in place 1024^2 FP16 with
+// a per-cell medium 12.3 -> 13.5 us.)
+__device__ __forceinline__ float wall_velocity(const StepParams& P, int w, int c) { return P.uw[2 * w + c]; }
+
 // momentum correction of the moving-wall bounce-back, 2 w_i rho0 (e_i . u_w) / c_s^2
 __device__ __forceinline__ float wall_term(const StepParams& P, int i, int w) {
-  return 6.0f * w_of(i) * P.rho0 * ((float)ex_of(i) * __ldg(P.uw + 2 * w) + (float)ey_of(i) * __ldg(P.uw + 2 * w + 1));
+  return 6.0f * w_of(i) * P.rho0 * ((float)ex_of(i) * wall_velocity(P, w, 0) + (float)ey_of(i) * wall_velocity(P, w, 1));
 }
 
 // e_i . u_w of wall w
 __device__ __forceinline__ float wall_dot(const StepParams& P, int i, int w) {
-  return __fadd_rn((float)ex_of(i) * __ldg(P.uw + 2 * w), (float)ey_of(i) * __ldg(P.uw + 2 * w + 1));
+  return __fadd_rn((float)ex_of(i) * wall_velocity(P, w, 0), (float)ey_of(i) * wall_velocity(P, w, 1));
 }
 
 // Halfway bounce-back: f_i(x) = f+_opp(i)(x) + 2 w_i rho0 (e_i . u_w) / c_s^2 with own = f+_opp(i)(x),
@@ -891,7 +898,7 @@ __device__ __forceinline__ void wall_node_from(const StepParams& P, const float 
   const float dr = (cb.phi - cn.phi) * cn.inv_phi;
   const float phip_b = mn.phip_dev + dr * (mn.phip_dev + P.p_rest);
   float eb[8], en[8];
-  feq_dev_d2q8(phip_b, __ldg(P.uw + 2 * w), __ldg(P.uw + 2 * w + 1), cb.inv_phi, P.rho0, eb);
+  feq_dev_d2q8(phip_b, wall_velocity(P, w, 0), wall_velocity(P, w, 1), cb.inv_phi, P.rho0, eb);
   feq_dev_d2q8(mn.phip_dev, mn.ux, mn.uy, cn.inv_phi, P.rho0, en);
 #pragma unroll
   for (int i = 0; i < 8; ++i) d[i] = eb[i] + dn[i] - en[i];
@@ -953,7 +960,7 @@ __device__ __forceinline__ void thermal_wall_node_from(const StepParams& P, cons
   wall_node_from<HET>(P, dn, x, y, xn, yn, w, P.ay + P.g_beta * Tn, d, uxn, uyn);
   const float Tb = P.Tdir[w] ? P.Tw[w] - P.T0 : Tn;
   float eb[5], en[5];
-  geq_dev(P, P.T0 + Tb, __ldg(P.uw + 2 * w), __ldg(P.uw + 2 * w + 1), eb);
+  geq_dev(P, P.T0 + Tb, wall_velocity(P, w, 0), wall_velocity(P, w, 1), eb);
   geq_dev(P, P.T0 + Tn, uxn, uyn, en);
 #pragma unroll
   for (int i = 0; i < 5; ++i) g[i] = eb[i] + gn[i] - en[i];

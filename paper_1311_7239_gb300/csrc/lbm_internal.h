@@ -15,7 +15,9 @@ constexpr int kResidualMaxBlocks = 2048;  // partial-sum slots of the residual r
 int record_error(int code, const char* msg);
 
 // Launch of a kernel that begins with wait_prerequisites(): it may be scheduled while the kernel
-// before it on the stream still runs.
+// before it on the stream still runs.  Such a kernel has no __restrict__ parameter (other than tables that
+// only the host writes) and reads what an earlier kernel may write by ordinary loads: a promise that the
+// memory does not change would let the compiler move the load up before the wait.
 template <class... P, class... A>
 inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchAttribute at;
