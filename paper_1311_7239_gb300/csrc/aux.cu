@@ -220,8 +220,10 @@ __global__ void k_export(const StepParams P, float* __restrict__ f, float* __res
     for (int i = 0; i < 5; ++i) g[i * dense + o] = gd[i] + 0.2f * P.T0;
 }
 
+// (the bounds: 40 and 48 registers, as without the walls' own load instruction)
 template <int PREC, bool HET, bool THERMAL>
-__global__ void k_macros(const StepParams P, float* __restrict__ p, float* __restrict__ ux, float* __restrict__ uy, float* __restrict__ Tout) {
+__global__ void __launch_bounds__(128, THERMAL ? 10 : 12) k_macros(const StepParams P, float* __restrict__ p, float* __restrict__ ux,
+                                                                   float* __restrict__ uy, float* __restrict__ Tout) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
   if (x >= P.nx) return;
@@ -280,10 +282,9 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
 
 // Pass 1: per-block partial sums of |u(t) - u(t-1)|^2 and |u(t)|^2 into partial[2 * block];
 // u(t-1) from the previous state (prev, gprev) or, if uprev is given, from its recorded
-// components (dense [2][ny][nx]).  (Three CTAs per SM: left to itself the compiler interleaves the loads
-// of the walls of several cells, 72 -> 128 registers.)
+// components (dense [2][ny][nx]).
 template <int PREC, bool HET, bool THERMAL>
-__global__ void __launch_bounds__(256, 3) k_residual_partial(const StepParams P, const void* prev, const void* gprev, const float* __restrict__ uprev,
+__global__ void k_residual_partial(const StepParams P, const void* prev, const void* gprev, const float* __restrict__ uprev,
                                    double* __restrict__ partial) {
   double num = 0.0, den = 0.0;
   const int64_t n = (int64_t)P.nx * P.ny;

@@ -741,9 +741,14 @@ __device__ __forceinline__ int64_t ip_source5(const StepParams& P, int x, int y,
 // Component c of the velocity of wall w.  lbm_set_walls may write it while a kernel that was launched
 // early is already resident: an ordinary load that stays behind wait_prerequisites(), and not one
 // through the read-only path, which takes memory that is constant for as long as the kernel lives.
-// (A volatile one is as safe and slower where the frame's cells bound a step: in place 1024^2 FP16 with
-// a per-cell medium 12.3 -> 13.5 us.)
-__device__ __forceinline__ float wall_velocity(const StepParams& P, int w, int c) { return P.uw[2 * w + c]; }
+// (Written as an instruction, so that it is not moved: as a plain load it let the compiler interleave
+// several cells, 72 -> 128 registers in the residual's kernel; a C++ volatile one passes by L1, and
+// steps bound by their frame cells slowed down, in place 1024^2 FP16 with a per-cell medium 12.3 -> 13.5 us.)
+__device__ __forceinline__ float wall_velocity(const StepParams& P, int w, int c) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(P.uw + 2 * w + c));
+  return v;
+}
 
 // momentum correction of the moving-wall bounce-back, 2 w_i rho0 (e_i . u_w) / c_s^2
 __device__ __forceinline__ float wall_term(const StepParams& P, int i, int w) {

@@ -229,6 +229,7 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE> {
   __device__ __forceinline__ void run(const March& M, int strip, int ya, int yb) {
     xs = march_x0<PREC, C>(strip, M.wrap);
     Ops::set_lane(xs, M.wrap);
+    Ops::read_wall();
     const int halo = march_halo<PREC, C>(M.wrap);
     const bool first = XE && !M.wrap && strip == 0, last = XE && !M.wrap && strip == M.strips - 1;
     out = (lane >= halo || first) && (lane < 32 - halo || last) && (!XE || x0 < P.nx);

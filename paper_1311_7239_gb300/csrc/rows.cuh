@@ -162,6 +162,12 @@ struct RowOps {
       outlet = kPressure && P.bc_x == BC_PRESSURE && x0 <= nx - 1 && x0 + C > nx - 1;
       cr = (nx - 1) & (C - 1);
       frame = PREC != PREC_FP32 && frame_cells();
+    }
+  }
+
+  // the side wall's velocity, after set_lane and once it may be read
+  __device__ __forceinline__ void read_wall() {
+    if constexpr (XE) {
       dot[0] = dot[1] = dot[2] = 0.0f;
       if (left || right) {
         const int w = left ? 0 : 1;

@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_consta
   Inner inner(P);
   Edge side(P);
   inner.set_lane(xs, M.wrap);
-  wait_prerequisites();  // (nothing above reads memory)
   side.set_lane(xs, M.wrap);
+  wait_prerequisites();  // (nothing above reads memory)
   const int x0 = inner.x0;
   const bool first = !M.wrap && strip == 0, last = !M.wrap && strip == M.strips - 1;
   const bool out = (first || lane * 2 >= M.halo) && (last || lane * 2 < kTileCells - M.halo) && x0 < nx;
@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_consta
     }
   }
   copy_commit();
+  side.read_wall();
   copy_wait<0>();
   __syncthreads();
 
