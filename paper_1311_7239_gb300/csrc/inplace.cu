@@ -346,6 +346,7 @@ __device__ __forceinline__ void ip_block(const StepParams& P, int frame_blocks, 
       float dc[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) dc[i] = d[i][c];
+      next_cell();
       const Coef cf = HET ? coef_of(P, f4_get(ph4, c), f4_get(k4, c), P.sv ? __ldg(P.sv + r0 + x0 + c) : P.s_v) : coef_uniform(P);
       float ay = P.ay;
       if (THERMAL) ay += P.g_beta * (g[0][c] + g[1][c] + g[2][c] + g[3][c] + g[4][c]);  // a = g beta (T - T0) j

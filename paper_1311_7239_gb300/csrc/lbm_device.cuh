@@ -236,6 +236,12 @@ __device__ __forceinline__ float rsqrt_normal(float x) {
 
 __device__ __forceinline__ float f4_get(const float4& v, int c) { return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w; }
 
+// Between the cells that a thread collides one after another: keeps the compiler from holding the
+// parameters, or a second cell's intermediate results, in registers across cells, which made the kernels
+// that are capped at 64 registers spill (bytes of spill stores: the in-place step that records u, FP32,
+// 144-168 -> 0 and 4096^2 208 -> 184 us; the in-place batches 48-72 -> 24-28).
+__device__ __forceinline__ void next_cell() { asm volatile("" ::: "memory"); }
+
 // Coefficients of a cell with porosity ph, permeability k and viscous rate sv (Eqs. 3-4, 13).
 __device__ __forceinline__ Coef coef_of(const StepParams& P, float ph, float k, float sv) {
   Coef c;
