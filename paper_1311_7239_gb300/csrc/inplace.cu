@@ -298,7 +298,7 @@ __device__ __forceinline__ void ip_block(const StepParams& P, int frame_blocks, 
 #pragma unroll
       for (int i = 0; i < 8; ++i) dp2[i] = S::w2f(w[i][h]);
       float2 ux, uy;
-      collide_pair(dp2, pair_coef_uniform(P.pc), f2(P.pc.u_hx), f2(P.pc.u_hy), P.pc, ux, uy);
+      collide_pair<false>(dp2, pair_coef_uniform(P.pc), f2(P.pc.u_hx), f2(P.pc.u_hy), P.pc, ux, uy);
       check += (fabsf(ux.x) + fabsf(uy.x)) + (fabsf(ux.y) + fabsf(uy.y));
       if (REC) record_u2(P, x0 + 2 * h, y, ux, uy);
 #pragma unroll

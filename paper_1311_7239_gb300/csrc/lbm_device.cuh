@@ -429,6 +429,11 @@ __device__ __forceinline__ PairCoef pair_coef_het(const StepParams& P, float2 ph
 }
 
 // hx, hy: phi a / 2 of the two cells.  d: in, stored pre-collision deviations; out, post-collision.
+// FTZ: the reciprocal and the root by rcp_normal and rsqrt_normal, which give the bits of fast_rcp and
+// rsqrtf for normal arguments (every float in range compared).  Fewer instructions (k_march 4096^2 FP16
+// 86 -> 81 us per step), but another schedule, in which k_step with a per-cell medium spills 60 bytes
+// instead of 24 (4096^2 FP16 110.0 -> 112.0 us) and the in-place step slows down (100.1 -> 102.1 us).
+template <bool FTZ = true>
 __device__ __forceinline__ void collide_pair(float2 d[8], const PairCoef& c, float2 hx, float2 hy, const PairConst& K, float2& ux,
                                              float2& uy) {
   // m = M d, Eq. 10 (as collide_d2q8)
@@ -447,8 +452,8 @@ __device__ __forceinline__ void collide_pair(float2 d[8], const PairCoef& c, flo
   const float2 vsq = fma2(vx, vx, mul2(vy, vy));
   const float2 vmag = mul2(vsq, make_float2(vsq.x > 0.0f ? rsqrtf(vsq.x) : 0.0f, vsq.y > 0.0f ? rsqrtf(vsq.y) : 0.0f));
   const float2 t = fma2(c.l1, vmag, c.l0sq);  // >= l0^2 >= 1/4
-  const float2 den = add2(c.l0, mul2(t, make_float2(rsqrt_normal(t.x), rsqrt_normal(t.y))));
-  const float2 inv = make_float2(rcp_normal(den.x), rcp_normal(den.y));
+  const float2 den = add2(c.l0, mul2(t, FTZ ? make_float2(rsqrt_normal(t.x), rsqrt_normal(t.y)) : make_float2(rsqrtf(t.x), rsqrtf(t.y))));
+  const float2 inv = FTZ ? make_float2(rcp_normal(den.x), rcp_normal(den.y)) : make_float2(fast_rcp(den.x), fast_rcp(den.y));
   ux = mul2(vx, inv);
   uy = mul2(vy, inv);
   const float2 umag = mul2(vmag, inv);

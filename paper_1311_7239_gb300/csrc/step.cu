@@ -63,8 +63,9 @@ __device__ void frame_step(const StepParams& P, const Frame& F, int k) {
 // form (two cells per 32-bit word) until each pair is collided, which halves the registers that
 // hold the gathered state.  A per-cell medium is read as float4 vectors of the four cells, issued
 // ahead of the populations, and turned into pair coefficients per pair; with the temperature
-// (uniform medium) the D2Q5 populations are gathered and collided the same way.
-template <int PREC, bool HET, bool THERMAL, int NT>
+// (uniform medium) the D2Q5 populations are gathered and collided the same way.  ONE: the step of one
+// lattice, not of a batch (see collide_pair's FTZ).
+template <int PREC, bool HET, bool THERMAL, int NT, bool ONE>
 __device__ __forceinline__ void step_item_words(const StepParams& P, const Tiling& tl, int item) {
   static_assert(!(HET && THERMAL), "the temperature step with a per-cell medium uses the scalar path");
   using S = Store<PREC>;
@@ -121,7 +122,7 @@ __device__ __forceinline__ void step_item_words(const StepParams& P, const Tilin
       const PairCoef c = pair_coef_het(P, h ? make_float2(ph4.z, ph4.w) : make_float2(ph4.x, ph4.y),
                                        h ? make_float2(k4.z, k4.w) : make_float2(k4.x, k4.y),
                                        h ? make_float2(sv4.z, sv4.w) : make_float2(sv4.x, sv4.y), hx, hy);
-      collide_pair(dp, c, hx, hy, P.pc, ux, uy);
+      collide_pair<!ONE>(dp, c, hx, hy, P.pc, ux, uy);
     } else if (THERMAL) {
       float2 gp[5];
 #pragma unroll
@@ -154,7 +155,7 @@ __device__ __forceinline__ void step_item_words(const StepParams& P, const Tilin
 // Work item `item` of one lattice, for CTAs of NT threads: items [0, frame_blocks) do the frame,
 // the rest cover the lattice row by row, gx items per row, and store every group that is not a
 // frame group.  Every thread of the CTA calls this with the same item (warp shuffles inside).
-template <int PREC, bool HET, bool THERMAL, int NT>
+template <int PREC, bool HET, bool THERMAL, int NT, bool ONE = false>
 __device__ __forceinline__ void step_item(const StepParams& P, const Tiling& tl, int item) {
   using S = Store<PREC>;
   using T = typename S::T;
@@ -165,7 +166,7 @@ __device__ __forceinline__ void step_item(const StepParams& P, const Tiling& tl,
     return;
   }
   if constexpr (PREC != PREC_FP32 && !(HET && THERMAL)) {
-    step_item_words<PREC, HET, THERMAL, NT>(P, tl, item);
+    step_item_words<PREC, HET, THERMAL, NT, ONE>(P, tl, item);
     return;
   }
   int x0, y;
@@ -291,7 +292,7 @@ template <int PREC, bool HET, bool THERMAL>
 __global__ void __launch_bounds__(kStepThreads, THERMAL ? (PREC != PREC_FP32 && HET ? 5 : 6) : 8) k_step(const StepParams P, Tiling tl) {
   launch_dependents();
   wait_prerequisites();
-  step_item<PREC, HET, THERMAL, kStepThreads>(P, tl, blockIdx.x);
+  step_item<PREC, HET, THERMAL, kStepThreads, true>(P, tl, blockIdx.x);
 }
 
 template <int PREC, bool HET, bool THERMAL>
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(NT, (PREC == PREC_BF16 ? 1024 : 896) / NT)
   Q.pc.hax = 0.5f * r.ax;
   Q.pc.hay = 0.5f * r.ay;
   if constexpr (PREC == PREC_FP32) step_item<PREC, true, false, NT>(Q, tl, item);
-  else step_item_words<PREC, true, false, NT>(Q, tl, item);
+  else step_item_words<PREC, true, false, NT, false>(Q, tl, item);
 }
 
 template <int PREC, int NT>
