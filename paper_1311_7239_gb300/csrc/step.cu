@@ -340,12 +340,13 @@ __device__ __forceinline__ void load_params(StepParams& sP, const StepParams* __
 }
 
 // Register caps (measured on a 512-lattice ensemble): the streaming rate follows the number of
-// resident warps, so the per-item form is held to 64 registers with FP32 storage (32 warps per SM,
-// a few bytes of spill) and to 80 with 16-bit storage (24 warps; its packed collision spills
+// resident warps, so the per-item form is held to 72 registers with FP32 storage (28 warps per SM; 128
+// lattices of 64..512 cells a side 143.7 us per step, 154.0 at 64, where the collision spills 100 bytes,
+// 152.9 at 80) and to 80 with 16-bit storage (24 warps; its packed collision spills
 // 200 bytes at 64 and runs 13 % slower), the persistent form to 85 (24 warps); uncapped they take
 // 72-108 registers and run 1.2-1.5x slower.  flat: the lattices' tiling (tiling_of).
 template <int PREC, int NT>
-__global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 1024 : 768) / NT) k_step_batch_items(const StepParams* __restrict__ Pd,
+__global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 896 : 768) / NT) k_step_batch_items(const StepParams* __restrict__ Pd,
                                                                                          const int64_t* __restrict__ item_start,
                                                                                          const int* __restrict__ item_lattice, int flat) {
   __shared__ StepParams sP;
@@ -360,12 +361,13 @@ __global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 1024 : 768) / NT) k_s
 // parameters, by value: the kernel's constant bank) supplies those and the collision constants, the
 // record of the item's lattice the fields that differ, so a main item starts its gathers without
 // staging the parameter set in shared memory and keeps the constants out of the registers.  Frame
-// items, which use every parameter, stage the lattice's set as the general form.  Register caps
-// (512-lattice ensemble): FP16 at 72 registers 122.1 GLUPS (117.7 at 64, 112.9 at 80; the staged
-// form 102.4), BF16 at 64 (113.4-114.7 at 64-80), FP32 at 72 (48 lattices 85.3 GLUPS, 81.7 at 64, which
-// its collision with written-out roundings spills).
+// items, which use every parameter, stage the lattice's set as the general form.  Register caps:
+// FP16 and BF16 at 72 registers (FP16, 512 lattices: 122.1 GLUPS, 117.7 at 64, 112.9 at 80, the staged
+// form 102.4; BF16, 128 lattices of 64..512 cells a side: 109.3 us per step, 114.2 at 64, 118.1 at 80),
+// FP32 at 64 (the same 128 lattices 138.4, 138.5 at 72; 8 lattices of 64..256, whose CTAs just fit the
+// chip at once, 5.9, 7.0 at 72).
 template <int PREC, int NT>
-__global__ void __launch_bounds__(NT, (PREC == PREC_BF16 ? 1024 : 896) / NT)
+__global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 1024 : 896) / NT)
     k_step_batch_items_shared(const StepParams U, const BatchRec* __restrict__ R, const StepParams* __restrict__ Pd,
                               const int64_t* __restrict__ item_start, const int* __restrict__ item_lattice, int flat) {
   launch_dependents();
