@@ -71,6 +71,7 @@ struct lbm_batch {
   MarchItem* pair_side = nullptr;
   MarchItem* pair_main = nullptr;
   int n_pair_side = 0, n_pair_main = 0;
+  bool pair_pressure = false;  // a lattice has pressure columns
   int cur = 0;
   int64_t steps = 0;
   int64_t cells = 0;
@@ -198,7 +199,7 @@ int launch_once(lbm_batch* b, int cur, cudaStream_t s) {
 }
 
 cudaError_t launch_pair(const lbm_batch* b, int cur, cudaStream_t s) {
-  return launch_march_batch(b->dp[cur], b->pair_side, b->n_pair_side, b->pair_main, b->n_pair_main, s);
+  return launch_march_batch(b->dp[cur], b->pair_side, b->n_pair_side, b->pair_main, b->n_pair_main, b->pair_pressure, s);
 }
 
 // Items of the pair kernels, if every lattice has a form that they handle and the batch is above the
@@ -212,6 +213,7 @@ int set_pairs(lbm_batch* b) {
   for (int d = 0; d < b->n; ++d) {
     if (!march_shape(b->hp[0][d], b->prec, true, false)) return LBM_OK;
     march_items(b->hp[0][d], d, side, main);
+    if (b->hp[0][d].bc_x == BC_PRESSURE) b->pair_pressure = true;
   }
   int rc = balloc(b, reinterpret_cast<void**>(&b->pair_side), side.size() * sizeof(MarchItem), "cudaMalloc(pair items)");
   if (rc == LBM_OK && !main.empty()) rc = balloc(b, reinterpret_cast<void**>(&b->pair_main), main.size() * sizeof(MarchItem), "cudaMalloc(pair items)");

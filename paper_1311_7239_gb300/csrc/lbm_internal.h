@@ -67,7 +67,8 @@ struct MarchItem {
   int lattice, strip, ya, yb, strips, wrap;
 };
 void march_items(const StepParams& P, int lattice, std::vector<MarchItem>& side, std::vector<MarchItem>& main);
-cudaError_t launch_march_batch(const StepParams* Pd, const MarchItem* side, int n_side, const MarchItem* main, int n_main, cudaStream_t s);
+cudaError_t launch_march_batch(const StepParams* Pd, const MarchItem* side, int n_side, const MarchItem* main, int n_main, bool pressure,
+                               cudaStream_t s);  // pressure: a lattice has pressure columns
 int tile_steps(const StepParams& P, int prec, bool het, bool thermal);
 cudaError_t launch_tile(const StepParams& P, int prec, bool het, bool thermal, int steps, cudaStream_t s);
 cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s);

@@ -56,9 +56,9 @@ __host__ __device__ inline int march_x0(int strip, bool wrap) {
 
 // One warp's march over the rows [ya, yb) of a strip.  XE: the strip has an x side (or, with 16-bit
 // storage, a frame group) within reach; YE: the rows have a y side within reach.
-template <int PREC, bool HET, bool THERMAL, int C, int STAGES, bool XE, bool YE>
-struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE> {
-  using Ops = RowOps<PREC, HET, THERMAL, C, XE, YE>;
+template <int PREC, bool HET, bool THERMAL, int C, int STAGES, bool XE, bool YE, bool PRESS = false>
+struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
+  using Ops = RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS>;
   using typename Ops::E;
   using typename Ops::V;
   using Ops::EDGE;
@@ -344,7 +344,7 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE> {
 // The warps at the sides: the bottom and top segments, then the strips with an x side in pieces of
 // `rows` rows.  A kernel of its own, so that the rules at the sides cost the main one no registers;
 // it lets the main kernel start at once (the two write different cells).
-template <int PREC, bool HET, bool THERMAL, int C, int STAGES>
+template <int PREC, bool HET, bool THERMAL, int C, int STAGES, bool PRESS>
 __global__ void __launch_bounds__(kMarchThreads) k_march_side(const __grid_constant__ StepParams P, const __grid_constant__ March M) {
   extern __shared__ __align__(16) char smem[];
   launch_dependents();
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kMarchThreads) k_march_side(const __grid_const
   const int ny = P.ny, sides = M.strips - (M.s1 - M.s0);
   if (item < 2 * M.strips) {
     const int top = item >= M.strips;
-    Marcher<PREC, HET, THERMAL, C, STAGES, true, true> m(P, buf);
+    Marcher<PREC, HET, THERMAL, C, STAGES, true, true, PRESS> m(P, buf);
     m.run(M, top ? item - M.strips : item, top ? ny - kMarchSide : 0, top ? ny : kMarchSide);
     return;
   }
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kMarchThreads) k_march_side(const __grid_const
   int strip = item - seg * sides;
   if (strip >= M.s0) strip += M.s1 - M.s0;
   const int ya = kMarchSide + seg * M.side_rows, yb = min(ya + M.side_rows, ny - kMarchSide);
-  Marcher<PREC, HET, THERMAL, C, STAGES, true, false> m(P, buf);
+  Marcher<PREC, HET, THERMAL, C, STAGES, true, false, PRESS> m(P, buf);
   m.run(M, strip, ya, yb);
 }
 
@@ -442,7 +442,10 @@ static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
   M.segs = (ny + M.rows - 1) / M.rows;
   M.side_segs = (ny + M.side_rows - 1) / M.side_rows;
   const size_t bytes = (kMarchThreads / 32) * STAGES * Marcher<PREC, HET, THERMAL, C, STAGES, false, false>::kStage;
-  auto side = k_march_side<PREC, HET, THERMAL, C, STAGES>;
+  auto side = k_march_side<PREC, HET, THERMAL, C, STAGES, false>;
+  if constexpr (PREC == PREC_FP32 && !THERMAL) {
+    if (P.bc_x == BC_PRESSURE) side = k_march_side<PREC, HET, THERMAL, C, STAGES, true>;
+  }
   auto main = k_march<PREC, HET, THERMAL, C, STAGES, CTAS>;
   cudaError_t e = cudaFuncSetAttribute(side, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(main, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -483,7 +486,7 @@ cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, 
 // --------------------------------------------------------------------------------------------
 constexpr int kBatchC = 2, kBatchStages = 3;
 
-template <bool SIDE>
+template <bool SIDE, bool PRESS>
 __global__ void __launch_bounds__(kMarchThreads, SIDE ? 1 : 4)
     k_march_batch(const StepParams* __restrict__ Pd, const MarchItem* __restrict__ items) {
   extern __shared__ __align__(16) char smem[];
@@ -504,10 +507,10 @@ __global__ void __launch_bounds__(kMarchThreads, SIDE ? 1 : 4)
       Inner m(sP, buf);
       m.run(M, it.strip, it.ya, it.yb);
     } else if (it.ya == 0 || it.yb == sP.ny) {
-      Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, true, true> m(sP, buf);
+      Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, true, true, PRESS> m(sP, buf);
       m.run(M, it.strip, it.ya, it.yb);
     } else {
-      Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, true, false> m(sP, buf);
+      Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, true, false, PRESS> m(sP, buf);
       m.run(M, it.strip, it.ya, it.yb);
     }
   }
@@ -534,10 +537,11 @@ void march_items(const StepParams& P, int lattice, std::vector<MarchItem>& side,
   pad(main);
 }
 
-cudaError_t launch_march_batch(const StepParams* Pd, const MarchItem* side, int n_side, const MarchItem* main, int n_main, cudaStream_t s) {
+cudaError_t launch_march_batch(const StepParams* Pd, const MarchItem* side, int n_side, const MarchItem* main, int n_main, bool pressure,
+                               cudaStream_t s) {
   const size_t bytes = (kMarchThreads / 32) * kBatchStages * Marcher<PREC_FP32, true, false, kBatchC, kBatchStages, false, false>::kStage;
-  auto sides = k_march_batch<true>;
-  auto inner = k_march_batch<false>;
+  auto sides = pressure ? k_march_batch<true, true> : k_march_batch<true, false>;
+  auto inner = k_march_batch<false, false>;
   cudaError_t e = cudaFuncSetAttribute(sides, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(inner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;

@@ -33,9 +33,9 @@ __host__ __device__ inline int tile_strips(int nx, int halo, bool wrap) {
 }
 __host__ __device__ inline int tile_x0(int strip, int halo, bool wrap) { return strip * tile_out(halo) - (wrap ? halo : 0); }
 
-template <int PREC, bool HET, bool THERMAL, bool EDGE>
-struct TileRow : RowOps<PREC, HET, THERMAL, 2, EDGE, EDGE> {
-  using Ops = RowOps<PREC, HET, THERMAL, 2, EDGE, EDGE>;
+template <int PREC, bool HET, bool THERMAL, bool EDGE, bool PRESS>
+struct TileRow : RowOps<PREC, HET, THERMAL, 2, EDGE, EDGE, PRESS> {
+  using Ops = RowOps<PREC, HET, THERMAL, 2, EDGE, EDGE, PRESS>;
   using typename Ops::E;
   using typename Ops::V;
   using Ops::lane;
@@ -96,11 +96,11 @@ struct TileRow : RowOps<PREC, HET, THERMAL, 2, EDGE, EDGE> {
   }
 };
 
-template <int PREC, bool HET, bool THERMAL>
+template <int PREC, bool HET, bool THERMAL, bool PRESS>
 __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_constant__ StepParams P, const __grid_constant__ Tile M) {
   extern __shared__ __align__(16) char smem[];
-  using Inner = TileRow<PREC, HET, THERMAL, false>;
-  using Edge = TileRow<PREC, HET, THERMAL, true>;
+  using Inner = TileRow<PREC, HET, THERMAL, false, false>;
+  using Edge = TileRow<PREC, HET, THERMAL, true, PRESS>;
   using E = typename Inner::E;
   using V = typename Inner::V;
   launch_dependents();
@@ -244,7 +244,10 @@ int tile_steps(const StepParams& P, int prec, bool het, bool thermal) {
 template <int PREC, bool HET, bool THERMAL>
 static cudaError_t launch_tile_t(const StepParams& P, const Tile& M, int prec, cudaStream_t s) {
   const size_t bytes = tile_bytes(prec, HET, THERMAL, M.height + 2 * M.halo);
-  auto fn = k_tile<PREC, HET, THERMAL>;
+  auto fn = k_tile<PREC, HET, THERMAL, false>;
+  if constexpr (PREC == PREC_FP32 && !THERMAL) {
+    if (P.bc_x == BC_PRESSURE) fn = k_tile<PREC, HET, THERMAL, true>;
+  }
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
   if (e != cudaSuccess) return e;
   return launch_early(fn, dim3(M.strips * ((P.ny + M.height - 1) / M.height)), dim3(kTileWarps * 32), bytes, s, P, M);
