@@ -86,6 +86,20 @@ __device__ __forceinline__ bool dbg_check(const StepParams& P, bool ok) {
 #endif
 }
 
+// The same for shared memory: what ends at `end` lies within the CTA's dynamic shared memory, from smem on.
+__device__ __forceinline__ bool dbg_shared(const StepParams& P, const char* smem, const void* end) {
+#ifdef LBM_DEBUG
+  uint32_t bytes;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+  return dbg_check(P, static_cast<const char*>(end) <= smem + bytes);
+#else
+  (void)P;
+  (void)smem;
+  (void)end;
+  return true;
+#endif
+}
+
 // Programmatic dependent launch: the kernels of a step sequence let the next one on the stream be
 // launched while they still run, and touch memory only after the one before has ended, which hides
 // the launch latency (launch_early on the host).

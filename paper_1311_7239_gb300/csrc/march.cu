@@ -72,6 +72,8 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
   using Ops::low;
   using Ops::high;
   using Ops::col;
+  using Ops::in_rows;
+  using Ops::in_cols;
   using Ops::shift;
   using Ops::collide_row;
   using Ops::pick;
@@ -104,7 +106,7 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
         dy = 0;
       }
     }
-    return static_cast<const E*>(heat ? P.gsrc : P.src) + (int64_t)i * P.plane + (int64_t)wrap_y(y + dy) * P.pitch;
+    return static_cast<const E*>(heat ? P.gsrc : P.src) + (int64_t)i * P.plane + (int64_t)in_rows(wrap_y(y + dy)) * P.pitch;
   }
 
   // Starts the copies of the rows that the pull into row r reads into a stage.
@@ -117,17 +119,17 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
         char* d = st + p * kRow + lane * C * (int)sizeof(E);
         if constexpr (PREC == PREC_FP32) {
 #pragma unroll
-          for (int c = 0; c < C; ++c) copy_async4(d + 4 * c, row + col(c));
+          for (int c = 0; c < C; ++c) copy_async4(d + 4 * c, row + in_cols(col(c), 1));
         } else {
-          copy_async8(d, row + col(0));  // (nx is a multiple of 4)
+          copy_async8(d, row + in_cols(col(0), C));  // (nx is a multiple of 4)
         }
       }
       if constexpr (HET) {
         char* d = st + kPlanes * kRow + lane * C * 4;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-          copy_async4(d + 4 * c, P.phi + (int64_t)y * P.pitch + col(c));
-          copy_async4(d + kMed + 4 * c, P.K + (int64_t)y * P.pitch + col(c));
+          copy_async4(d + 4 * c, P.phi + (int64_t)in_rows(y) * P.pitch + in_cols(col(c), 1));
+          copy_async4(d + kMed + 4 * c, P.K + (int64_t)in_rows(y) * P.pitch + in_cols(col(c), 1));
         }
       }
     } else if constexpr (EDGE) {
@@ -136,7 +138,7 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
         const int q = j * 32 + lane, p = q / kChunks;
         if ((j + 1) * 32 <= kPlanes * kChunks || p < kPlanes) {
           const int x = min(xs + (q - p * kChunks) * (16 / (int)sizeof(E)), P.pitch - 16 / (int)sizeof(E));
-          copy_async16(st + q * 16, source(p, y) + x);
+          copy_async16(st + q * 16, source(p, y) + in_cols(x, 16 / (int)sizeof(E)));
         }
       }
       if constexpr (HET) {
@@ -144,10 +146,10 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
         for (int j = 0; j < 2 * kMedChunks / 32; ++j) {
           const int q = j * 32 + lane, p = q / kMedChunks;
           const int x = min(xs + (q - p * kMedChunks) * 4, P.pitch - 4);
-          copy_async16(st + kPlanes * kRow + q * 16, (p ? P.K : P.phi) + (int64_t)y * P.pitch + x);
+          copy_async16(st + kPlanes * kRow + q * 16, (p ? P.K : P.phi) + (int64_t)in_rows(y) * P.pitch + in_cols(x, 4));
         }
       }
-    } else {
+    } else if (dbg_check(P, r >= 1 && r < P.ny - 1 && xs >= 0 && xs + 32 * C <= P.pitch)) {
       // 16-byte units from the start of the flow or temperature planes in 32 bits (march_takes checks):
       // the lane's part `at` of each copy is kept, the row's part is the same for the warp
       const uint32_t row = (uint32_t)r * ((uint32_t)P.pitch * (uint32_t)sizeof(E) / 16);
@@ -155,7 +157,10 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
 #pragma unroll
       for (int j = 0; j < kCopies; ++j) {
         const char* base = static_cast<const char*>(32 * j >= 8 * kChunks ? P.gsrc : P.src);
-        if ((j + 1) * 32 <= kPlanes * kChunks || lane < kPlanes * kChunks - j * 32) copy_async16(d + j * 512, base + (uint64_t)(at[j] + row) * 16);
+        const uint32_t unit = at[j] + row;
+        if (((j + 1) * 32 <= kPlanes * kChunks || lane < kPlanes * kChunks - j * 32) &&
+            dbg_check(P, ((uint64_t)unit + 1) * 16 <= (32 * j >= 8 * kChunks ? 5 : 8) * (uint64_t)P.plane * sizeof(E)))
+          copy_async16(d + j * 512, base + (uint64_t)unit * 16);
       }
       if constexpr (HET) {
         const uint32_t mrow = (uint32_t)r * ((uint32_t)P.pitch / 4);
@@ -163,7 +168,8 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
         for (int j = 0; j < 2 * kMedChunks / 32; ++j) {
           const int q = j * 32 + lane, p = q / kMedChunks;
           const uint32_t x = (uint32_t)(xs / 4 + q - p * kMedChunks) + mrow;
-          copy_async16(st + kPlanes * kRow + q * 16, reinterpret_cast<const char*>(p ? P.K : P.phi) + (uint64_t)x * 16);
+          if (dbg_check(P, ((int64_t)x + 1) * 4 <= P.plane))
+            copy_async16(st + kPlanes * kRow + q * 16, reinterpret_cast<const char*>(p ? P.K : P.phi) + (uint64_t)x * 16);
         }
       }
     }
@@ -186,7 +192,7 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
   // the side columns' own populations of row r (prefetched: plain loads, used one row later)
   __device__ __forceinline__ void fetch_own(int r) {
     if (XE && (left || right)) {
-      const int y = wrap_y(r);
+      const int y = in_rows(wrap_y(r));
       const E* own = static_cast<const E*>(P.src) + (int64_t)y * P.pitch + (left ? 0 : P.nx - 1);
       e[0] = raw_bits<PREC>(own + (left ? 2 : 0) * P.plane);
       e[1] = raw_bits<PREC>(own + (left ? 6 : 7) * P.plane);
@@ -199,6 +205,7 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
   }
 
   __device__ __forceinline__ void store(int y, V w[8], V gw[5]) const {
+    if (!dbg_check(P, y >= 0 && y < P.ny && x0 >= 0 && x0 + C <= P.pitch)) return;
     if (XE && x0 + C > P.nx) {  // row padding holds zeros
 #pragma unroll
       for (int c = 0; c < C; ++c) {
@@ -227,6 +234,8 @@ struct Marcher : RowOps<PREC, HET, THERMAL, C, XE, YE, PRESS> {
   }
 
   __device__ __forceinline__ void run(const March& M, int strip, int ya, int yb) {
+    if (!dbg_check(P, strip >= 0 && strip < M.strips && ya >= 0 && yb <= P.ny)) return;
+    if (!dbg_shared(P, buf - (threadIdx.x >> 5) * (STAGES * kStage), buf + STAGES * kStage)) return;
     xs = march_x0<PREC, C>(strip, M.wrap);
     Ops::set_lane(xs, M.wrap);
     Ops::read_wall();

@@ -190,6 +190,11 @@ struct RowOps {
   __device__ __forceinline__ int wrap_y(int y) const { return !YE ? y : y < 0 ? y + P.ny : (y >= P.ny ? y - P.ny : y); }
   __device__ __forceinline__ bool low(int y) const { return YE && P.bc_y == BC_WALL && y == 0; }
   __device__ __forceinline__ bool high(int y) const { return YE && P.bc_y == BC_WALL && y == P.ny - 1; }
+  // a row of the lattice; n columns, from a multiple of n on, of a row with its padding (debug builds check)
+  __device__ __forceinline__ int in_rows(int y) const { return dbg_check(P, y >= 0 && y < P.ny) ? y : 0; }
+  __device__ __forceinline__ int in_cols(int x, int n) const {
+    return dbg_check(P, x >= 0 && x + n <= P.pitch && (x & (n - 1)) == 0) ? x : 0;
+  }
   // column of the lane's cell c in memory; where the cell is never part of a stored result, some column
   // that keeps the alignment of the lane's first cell
   __device__ __forceinline__ int col(int c) const {
@@ -305,9 +310,9 @@ struct RowOps {
         patch_cell(cb, y, e, eg, db, gb);
         Coef ma, mb;
         if constexpr (HET) {
-          const float* sv = P.sv ? P.sv + (int64_t)y * P.pitch : nullptr;
-          ma = coef_of(P, ph[ca], k[ca], sv ? __ldg(sv + col(ca)) : P.s_v);
-          mb = coef_of(P, ph[cb], k[cb], sv ? __ldg(sv + col(cb)) : P.s_v);
+          const float* sv = P.sv ? P.sv + (int64_t)in_rows(y) * P.pitch : nullptr;
+          ma = coef_of(P, ph[ca], k[ca], sv ? __ldg(sv + in_cols(col(ca), 1)) : P.s_v);
+          mb = coef_of(P, ph[cb], k[cb], sv ? __ldg(sv + in_cols(col(cb), 1)) : P.s_v);
         } else {
           ma = mb = coef_uniform(P);
         }
@@ -347,8 +352,8 @@ struct RowOps {
 
   // viscous rates of the lane's cells a, a + 1 of row y
   __device__ __forceinline__ float2 rates(int y, int a) const {
-    const float* sv = P.sv + (int64_t)y * P.pitch;
-    return make_float2(__ldg(sv + col(a)), __ldg(sv + col(a + 1)));
+    const float* sv = P.sv + (int64_t)in_rows(y) * P.pitch;
+    return make_float2(__ldg(sv + in_cols(col(a), 1)), __ldg(sv + in_cols(col(a + 1), 1)));
   }
 
   // Collision of the lane's cells of row y, in place; returns the sum of |u| over the cells.

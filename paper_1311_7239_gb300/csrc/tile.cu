@@ -122,10 +122,11 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_consta
   inner.set_lane(xs, M.wrap);
   side.set_lane(xs, M.wrap);
   wait_prerequisites();  // (nothing above reads memory)
+  if (!dbg_check(P, ya < yb && M.steps >= 1 && M.steps <= M.halo) || !dbg_shared(P, smem, med + (HET ? rows * 2 * kTileCells : 0))) return;
   const int x0 = inner.x0;
   const bool first = !M.wrap && strip == 0, last = !M.wrap && strip == M.strips - 1;
   const bool out = (first || lane * 2 >= M.halo) && (last || lane * 2 < kTileCells - M.halo) && x0 < nx;
-  auto memory_row = [&](int y) { return y < 0 ? y + ny : (y >= ny ? y - ny : y); };
+  auto memory_row = [&](int y) { return side.in_rows(y < 0 ? y + ny : (y >= ny ? y - ny : y)); };
 
   // the tile (columns past the lattice are clamped: never part of a stored result)
   if constexpr (HET) {
@@ -133,8 +134,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_consta
       const int64_t o = (int64_t)memory_row(y0 + j) * P.pitch;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        med[j * 2 * kTileCells + lane * 2 + c] = __ldg(P.phi + o + side.col(c));
-        med[j * 2 * kTileCells + kTileCells + lane * 2 + c] = __ldg(P.K + o + side.col(c));
+        med[j * 2 * kTileCells + lane * 2 + c] = __ldg(P.phi + o + side.in_cols(side.col(c), 1));
+        med[j * 2 * kTileCells + kTileCells + lane * 2 + c] = __ldg(P.K + o + side.in_cols(side.col(c), 1));
       }
     }
   }
@@ -146,13 +147,13 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_consta
     for (int p = 0; p < Inner::kPlanes; ++p) {
       const E* row = (p >= 8 ? static_cast<const E*>(P.gsrc) + (p - 8) * P.plane : static_cast<const E*>(P.src) + p * P.plane) + o;
       if (!side.slow) {
-        if constexpr (PREC == PREC_FP32) copy_async8(d + p * Inner::kSpan, row + xl);
-        else copy_async4(d + p * Inner::kSpan, row + xl);
+        if constexpr (PREC == PREC_FP32) copy_async8(d + p * Inner::kSpan, row + side.in_cols(xl, 2));
+        else copy_async4(d + p * Inner::kSpan, row + side.in_cols(xl, 2));
       } else if constexpr (PREC == PREC_FP32) {
-        copy_async4(d + p * Inner::kSpan, row + side.col(0));
-        copy_async4(d + p * Inner::kSpan + 4, row + side.col(1));
+        copy_async4(d + p * Inner::kSpan, row + side.in_cols(side.col(0), 1));
+        copy_async4(d + p * Inner::kSpan + 4, row + side.in_cols(side.col(1), 1));
       } else {
-        copy_async4(d + p * Inner::kSpan, row + min(side.col(0), P.pitch - 2));  // (nx is a multiple of 4)
+        copy_async4(d + p * Inner::kSpan, row + side.in_cols(min(side.col(0), P.pitch - 2), 2));  // (nx is a multiple of 4)
       }
     }
   }
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_consta
     const int reach = M.steps - s;
     const int lo = (walls ? max(ya - reach, 0) : ya - reach) - y0, hi = (walls ? min(yb + reach, ny) : yb + reach) - y0;
     for (int j = lo + warp; j < hi; j += kTileWarps) {
+      if (!dbg_check(P, j >= 0 && j < rows)) continue;
       const int y = memory_row(y0 + j);
       V w[8], gw[5];
       const char* row = in + j * Inner::kRow;
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) k_tile(const __grid_consta
 #pragma unroll
           for (int p = 0; p < 5; ++p) store_cells<PREC, 2>(reinterpret_cast<E*>(d + (8 + p) * Inner::kSpan), gw[p]);
         }
-      } else if (out) {
+      } else if (out && dbg_check(P, x0 >= 0 && x0 + 2 <= P.pitch)) {
         if (x0 + 1 >= nx) {  // row padding holds zeros
 #pragma unroll
           for (int p = 0; p < 8; ++p) put_bits<PREC, 2>(w[p], 1, 0u);
