@@ -138,6 +138,7 @@ int set_launch(lbm_batch* b, int nt, int ctas_per_sm) {
     total += b->inplace ? inplace_items((int)c.nx, (int)c.ny, (int)c.bc_x, (int)c.bc_y)
                         : batch_items((int)c.nx, (int)c.ny, (int)c.bc_y, nt, b->flat);
   }
+  LBM_BCUDA(cudaStreamSynchronize(b->stream), "stream synchronize");  // (steps in flight read the tables)
   LBM_BCUDA(cudaMemcpy(b->item_start, start.data(), b->n * sizeof(int64_t), cudaMemcpyHostToDevice), "copy of the item table");
   b->total_items = total;
   b->nt = nt;
@@ -152,7 +153,6 @@ int set_launch(lbm_batch* b, int nt, int ctas_per_sm) {
   if (ctas_per_sm == 0) {  // one CTA per work item
     if (total > 0x7fffffffLL) return fail_msg(LBM_EINVAL, "too many work items for one CTA per item");
     if (b->item_lattice_cap < total) {
-      cudaStreamSynchronize(b->stream);
       cudaFree(b->item_lattice);
       b->bytes -= (uint64_t)b->item_lattice_cap * sizeof(int);
       b->item_lattice = nullptr;
