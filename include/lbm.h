@@ -264,7 +264,8 @@ LBM_API int lbm_nusselt(lbm_ctx* ctx, int side, double* nu);
  * Batched ensembles: n independent isothermal lattices, each with its own lbm_config (size,
  * boundaries, parameters, medium; one storage precision for all), advanced together by one
  * launch per time step over the concatenated work items of all lattices (one CTA per item, CTAs
- * of a few items, or a persistent grid: lbm_batch_set_launch, lbm_batch_tune), with
+ * of a few items, or a persistent grid: lbm_batch_set_launch, lbm_batch_tune), or two kernels per
+ * two steps (lbm_batch_set_steps_per_launch), with
  * runs of 32 steps replayed as a captured CUDA graph.  The batch runs on cfgs[0].stream (NULL:
  * a stream of its own).  Every lattice keeps per-cell medium fields (8 B per cell).  All lattices
  * use one streaming form: LBM_STREAM_AB (two population pools), or LBM_STREAM_INPLACE (one pool,
@@ -282,14 +283,16 @@ LBM_API void lbm_batch_destroy(lbm_batch* b);
 LBM_API int lbm_batch_set_medium(lbm_batch* b, int d, const float* eps, const float* K);
 /* Equilibrium initial state of lattice d (d = -1: all), as lbm_init_equilibrium. */
 LBM_API int lbm_batch_init_equilibrium(lbm_batch* b, int d, double p0, double ux0, double uy0, int phi_p_uniform);
-/* Advance every lattice by n steps with the batched kernel (one launch per step for the batch). */
+/* Advance every lattice by n steps with the batched kernels: one launch per step for the batch, or
+ * two kernels per two steps and a single one for an odd last step (the same bits). */
 LBM_API int lbm_batch_step(lbm_batch* b, int n);
 /* The same n steps run lattice by lattice with the single-lattice kernel (for comparison). */
 LBM_API int lbm_batch_step_each(lbm_batch* b, int n);
 /* Launch shape of the batched kernel: threads per CTA (64, 128, 256) and CTAs per SM: 0 = one CTA
  * per work item (a lattice table of 4 bytes per item is kept on the device), 1..32 = a persistent
  * grid of SMs x k CTAs, k lowered to the kernel's occupancy limit so that every CTA is resident.
- * In-place batches take (128, 0) only (EINVAL otherwise). */
+ * In-place batches take (128, 0) only (EINVAL otherwise).  Choosing a shape, items per CTA or a
+ * tiling makes lbm_batch_step take its steps with that kernel, one per launch. */
 LBM_API int lbm_batch_set_launch(lbm_batch* b, int threads_per_cta, int ctas_per_sm);
 LBM_API int lbm_batch_get_launch(const lbm_batch* b, int* threads_per_cta, int* ctas_per_sm);
 /* Work items per CTA when ctas_per_sm = 0: 1 (the default) = one CTA per work item; 2, 4 or 8 = CTAs
@@ -310,10 +313,18 @@ LBM_API int lbm_batch_get_items_per_cta(const lbm_batch* b, int* items_per_cta);
 #define LBM_TILING_FLAT 1
 LBM_API int lbm_batch_set_tiling(lbm_batch* b, int tiling);
 LBM_API int lbm_batch_get_tiling(const lbm_batch* b, int* tiling);
+/* Steps per launch of lbm_batch_step: 2 (the default where available: A-B batches of FP32 storage above
+ * 100 MiB with at least 120000 cells per lattice on average, sides of 16 or more, no LBM_NEE sides)
+ * or 1, in the launch shape above.  EINVAL for 2 where it is not available. */
+LBM_API int lbm_batch_set_steps_per_launch(lbm_batch* b, int steps);
+LBM_API int lbm_batch_get_steps_per_launch(const lbm_batch* b, int* steps);
 /* Time `steps` steps for every launch shape (threads per CTA 64 / 128 / 256; one CTA per work item,
- * CTAs of 2 or 4 work items, persistent grids of 1..16 CTAs per SM) and tiling on a copy of the
- * current state, keep the fastest, restore the state; outputs may be NULL (the chosen tiling and
- * work items per CTA: lbm_batch_get_tiling, lbm_batch_get_items_per_cta).  Waits for the stream. */
+ * CTAs of 2 or 4 work items, persistent grids of 1..16 CTAs per SM) and tiling, and two steps per
+ * launch where available, on a copy of the current state, keep the fastest, restore the state;
+ * outputs may be NULL (the chosen tiling, work items per CTA and steps per launch:
+ * lbm_batch_get_tiling, lbm_batch_get_items_per_cta, lbm_batch_get_steps_per_launch; with two steps
+ * per launch, the shape is the one for an odd last step and ms_per_step that of the pairs).  Waits
+ * for the stream. */
 LBM_API int lbm_batch_tune(lbm_batch* b, int steps, int* threads_per_cta, int* ctas_per_sm, float* ms_per_step);
 /* Read-outs of lattice d (float32 [ny_d][nx_d] / [8][ny_d][nx_d], host or device). */
 LBM_API int lbm_batch_macros(lbm_batch* b, int d, float* p, float* ux, float* uy);

@@ -67,7 +67,9 @@ struct lbm_batch {
   // fields that differ (one array per buffer parity) for the per-item kernel
   bool shared_consts = false;
   BatchRec* rec[2] = {nullptr, nullptr};
-  // A-B FP32 batches above the size of L2: work items of the kernels that take two steps per pass
+  // A-B FP32 batches above the size of L2: work items of the kernels that take two steps per pass, and
+  // whether lbm_batch_step uses them (until a launch shape of the single steps is chosen)
+  bool pairs = false;
   MarchItem* pair_side = nullptr;
   MarchItem* pair_main = nullptr;
   int n_pair_side = 0, n_pair_main = 0;
@@ -223,6 +225,7 @@ int set_pairs(lbm_batch* b) {
     LBM_BCUDA(cudaMemcpy(b->pair_main, main.data(), main.size() * sizeof(MarchItem), cudaMemcpyHostToDevice), "copy of the pair items");
   b->n_pair_side = (int)side.size();
   b->n_pair_main = (int)main.size();
+  b->pairs = true;
   return LBM_OK;
 }
 
@@ -230,9 +233,8 @@ int capture(lbm_batch* b, int cur) {
   if (!b->capture_stream) LBM_BCUDA(cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking), "cudaStreamCreate");
   LBM_BCUDA(cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
   cudaError_t le = cudaSuccess;
-  const bool pairs = b->n_pair_side > 0;
-  for (int k = 0; k < (pairs ? kBatchGraphSteps / 2 : kBatchGraphSteps) && le == cudaSuccess; ++k)
-    le = pairs ? launch_pair(b, cur ^ (k & 1), b->capture_stream) : launch_batch(b, cur ^ (k & 1), b->capture_stream);
+  for (int k = 0; k < (b->pairs ? kBatchGraphSteps / 2 : kBatchGraphSteps) && le == cudaSuccess; ++k)
+    le = b->pairs ? launch_pair(b, cur ^ (k & 1), b->capture_stream) : launch_batch(b, cur ^ (k & 1), b->capture_stream);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(b->capture_stream, &g);
   if (le != cudaSuccess || e != cudaSuccess) {
@@ -496,7 +498,7 @@ int lbm_batch_step(lbm_batch* b, int n) {
     b->steps += kBatchGraphSteps;
     n -= kBatchGraphSteps;
   }
-  for (; b->n_pair_side > 0 && n > 1; n -= 2) {
+  for (; b->pairs && n > 1; n -= 2) {
     LBM_BCUDA(launch_pair(b, b->cur, b->stream), "batched step kernels");
     b->cur ^= 1;
     b->steps += 2;
@@ -529,7 +531,9 @@ int lbm_batch_step_each(lbm_batch* b, int n) {
 
 int lbm_batch_set_launch(lbm_batch* b, int threads_per_cta, int ctas_per_sm) {
   if (!b) return fail_msg(LBM_EINVAL, "null batch");
-  return set_launch(b, threads_per_cta, ctas_per_sm);
+  const int rc = set_launch(b, threads_per_cta, ctas_per_sm);
+  if (rc == LBM_OK) b->pairs = false;
+  return rc;
 }
 
 int lbm_batch_get_launch(const lbm_batch* b, int* threads_per_cta, int* ctas_per_sm) {
@@ -548,6 +552,7 @@ int lbm_batch_set_items_per_cta(lbm_batch* b, int items_per_cta) {
   b->items_per_cta = items_per_cta;
   const int rc = set_launch(b, b->nt, b->ctas_per_sm);
   if (rc) b->items_per_cta = old;
+  else b->pairs = false;
   return rc;
 }
 
@@ -566,7 +571,23 @@ int lbm_batch_set_tiling(lbm_batch* b, int tiling) {
   b->flat = tiling == LBM_TILING_FLAT ? 1 : 0;
   const int rc = set_launch(b, b->nt, b->ctas_per_sm);
   if (rc) b->flat = old;
+  else b->pairs = false;
   return rc;
+}
+
+int lbm_batch_set_steps_per_launch(lbm_batch* b, int steps) {
+  if (!b) return fail_msg(LBM_EINVAL, "null batch");
+  if (steps != 1 && !(steps == 2 && b->n_pair_side > 0))
+    return fail_msg(LBM_EINVAL, "steps per launch must be 1, or 2 in a batch that takes steps in pairs");
+  if (b->pairs != (steps == 2)) drop_graphs(b);
+  b->pairs = steps == 2;
+  return LBM_OK;
+}
+
+int lbm_batch_get_steps_per_launch(const lbm_batch* b, int* steps) {
+  if (!b || !steps) return fail_msg(LBM_EINVAL, "null argument");
+  *steps = b->pairs ? 2 : 1;
+  return LBM_OK;
 }
 
 int lbm_batch_get_tiling(const lbm_batch* b, int* tiling) {
@@ -621,6 +642,24 @@ int lbm_batch_tune(lbm_batch* b, int steps, int* threads_per_cta, int* ctas_per_
         best_ipc = ipc[c];
       }
     }
+  bool best_pairs = false;
+  if (rc == LBM_OK && b->n_pair_side > 0) {  // two steps per launch, where the batch has that form
+    const int n = (steps + 1) / 2;
+    cudaError_t le = launch_pair(b, b->cur, b->stream);  // warm-up
+    cudaEventRecord(e0, b->stream);
+    for (int s = 0; s < n && le == cudaSuccess; ++s) le = launch_pair(b, b->cur ^ ((s + 1) & 1), b->stream);
+    cudaEventRecord(e1, b->stream);
+    cudaEventSynchronize(e1);
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    ms /= 2 * n;
+    if (le != cudaSuccess) {
+      rc = fail_msg(LBM_ECUDA, "batched step kernels");
+    } else if (ms < best) {
+      best = ms;
+      best_pairs = true;
+    }
+  }
   cudaMemcpyAsync(live, save, pool_bytes, cudaMemcpyDeviceToDevice, b->stream);
   cudaStreamSynchronize(b->stream);
   cudaFree(save);
@@ -630,6 +669,7 @@ int lbm_batch_tune(lbm_batch* b, int steps, int* threads_per_cta, int* ctas_per_
   b->flat = best_flat;
   b->items_per_cta = best_ipc;
   if ((rc = set_launch(b, best_nt, best_k))) return rc;
+  b->pairs = best_pairs;
   if (threads_per_cta) *threads_per_cta = best_nt;
   if (ctas_per_sm) *ctas_per_sm = best_k;
   if (ms_per_step) *ms_per_step = best;

@@ -114,6 +114,8 @@ SIGNATURES = {
     "lbm_batch_get_items_per_cta": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int)]),
     "lbm_batch_set_tiling": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
     "lbm_batch_get_tiling": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int)]),
+    "lbm_batch_set_steps_per_launch": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
+    "lbm_batch_get_steps_per_launch": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int)]),
     "lbm_batch_tune": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                       ctypes.POINTER(ctypes.c_float)]),
     "lbm_batch_macros": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, _f32p, _f32p, _f32p]),
@@ -433,15 +435,24 @@ class Batch:
         _check(lib().lbm_batch_get_tiling(self._h, ctypes.byref(t)), "lbm_batch_get_tiling")
         return t.value
 
+    def set_steps_per_launch(self, steps):
+        """1, or 2 where the batch can take its steps in pairs (``LbmError`` otherwise)."""
+        _check(lib().lbm_batch_set_steps_per_launch(self._h, int(steps)), "lbm_batch_set_steps_per_launch")
+
+    def get_steps_per_launch(self):
+        k = ctypes.c_int()
+        _check(lib().lbm_batch_get_steps_per_launch(self._h, ctypes.byref(k)), "lbm_batch_get_steps_per_launch")
+        return k.value
+
     def tune(self, steps=20):
         a, b, ms = ctypes.c_int(), ctypes.c_int(), ctypes.c_float()
         _check(lib().lbm_batch_tune(self._h, int(steps), ctypes.byref(a), ctypes.byref(b), ctypes.byref(ms)), "lbm_batch_tune")
         return a.value, b.value, ms.value
 
     def tune_cached(self, path=None, steps=20):
-        """Launch shape, work items per CTA and tiling from a JSON cache on disk (keyed by GPU, storage
-        precision, lattice count and total cells rounded to a power of two); a miss runs ``tune`` and
-        records the result."""
+        """Launch shape, work items per CTA, tiling and steps per launch from a JSON cache on disk (keyed by
+        GPU, storage precision, lattice count and total cells rounded to a power of two); a miss runs
+        ``tune`` and records the result."""
         import json
 
         import torch
@@ -456,13 +467,21 @@ class Batch:
             cache = {}
         if key in cache:
             nt, k = cache[key]["threads_per_cta"], cache[key]["ctas_per_sm"]
+            # (an entry without it was timed before there were pairs: the batch keeps its own choice)
+            pairs = cache[key].get("steps_per_launch", self.get_steps_per_launch()) == 2
             self.set_tiling(cache[key].get("tiling", TILING_FLAT))
             self.set_items_per_cta(cache[key].get("items_per_cta", 1))
             self.set_launch(nt, k)
+            if pairs:
+                try:
+                    self.set_steps_per_launch(2)
+                except LbmError as e:  # timed on a batch that has them; this one does not
+                    if e.code != EINVAL:
+                        raise
             return nt, k, cache[key]["ms_per_step"], True
         nt, k, ms = self.tune(steps)
         cache[key] = {"threads_per_cta": nt, "ctas_per_sm": k, "tiling": self.get_tiling(), "items_per_cta": self.get_items_per_cta(),
-                      "ms_per_step": ms}
+                      "steps_per_launch": self.get_steps_per_launch(), "ms_per_step": ms}
         os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
         tmp = path + ".tmp"
         with open(tmp, "w") as fh:
