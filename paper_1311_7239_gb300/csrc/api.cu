@@ -910,11 +910,12 @@ void ws_release(lbm_ctx* c) {
   c->ws_bytes = 0;
 }
 
-// The adjoint workspace, `bytes` long: the one kept from an earlier call when its size matches, else a
-// new one.  A single allocation: one per buffer took 3.7 ms of a 16 ms gradient (T = 100, 2048 x 1024)
-// to make and free.  Callers synchronise before the workspace changes hands.
+// The adjoint workspace, at least `bytes` long: the one kept from an earlier call when that is large
+// enough and not more than twice the size (calls whose T changes a little share one), else a new one.
+// A single allocation: one per buffer took 3.7 ms of a 16 ms gradient (T = 100, 2048 x 1024) to make and
+// free.  Callers synchronise before the workspace changes hands.
 int ws_reserve(lbm_ctx* c, size_t bytes) {
-  if (c->ws && c->ws_bytes == bytes) return LBM_OK;
+  if (c->ws && c->ws_bytes >= bytes && c->ws_bytes / 2 <= bytes) return LBM_OK;
   ws_release(c);
   const int rc = dev_alloc(c, reinterpret_cast<void**>(&c->ws), bytes, "cudaMalloc(adjoint workspace)");
   if (rc == LBM_OK) c->ws_bytes = bytes;
