@@ -32,14 +32,13 @@ PREC = {"fp32": 0, "fp16": 1, "bf16": 2}
 BYTES_PER_LU = {"fp32": 64, "fp16": 32, "bf16": 32}
 
 
-def steps_per_pass(prec, cells, populations=8, plain=True, sides="halfway"):
-    """Time steps that one pass over the populations takes (A-B streaming): two where the state is larger
-    than L2 (plain: no per-cell medium and no temperature), so that an update moves half the bytes."""
-    state = 2 * populations * cells * (4 if prec == "fp32" else 2)
-    if sides != "halfway":
-        return 1
-    return 2 if state >= (100 << 20 if prec == "fp32" else 120 << 20) and (plain or prec == "fp32") else 1
-
+def passes_per_step(lat, steps):
+    """Passes over the populations in memory per time step of lat.step(steps): 1, about 1/2 where a launch
+    takes two steps, None where it takes four on a tile in shared memory (a lattice that L2 holds)."""
+    k, _ = lat.step_plan(steps)
+    if k > 2:
+        return None
+    return 1.0 if k == 1 else (steps - (steps - 1) // 2) / steps
 
 
 def max_over_ranks(value, dist, device):
@@ -65,7 +64,9 @@ def cavity_params(L):
     return dict(nu=lid * L / 100.0, phi=0.4, K=1e-3 * L * L, lid=lid)
 
 
-KERNEL_SOURCES = {"k_step": ("lbm_device.cuh", "tiles.cuh", "step.cu"), "k_step_ip": ("lbm_device.cuh", "inplace.cu")}
+KERNEL_SOURCES = {"k_step": ("lbm_device.cuh", "tiles.cuh", "step.cu"), "k_step_ip": ("lbm_device.cuh", "inplace.cu"),
+                  "k_march": ("lbm_device.cuh", "tiles.cuh", "rows.cuh", "march.cu"),
+                  "k_tile": ("lbm_device.cuh", "tiles.cuh", "rows.cuh", "tile.cu")}
 
 
 def source_hash(kernel="k_step"):
@@ -79,14 +80,15 @@ def source_hash(kernel="k_step"):
     return h.hexdigest()[:16]
 
 
-def traffic_for(kernel_key):
-    """DRAM bytes per launch from a committed ncu capture, if it was taken on the current sources."""
+def traffic_for(kernel, key):
+    """DRAM bytes per launch (k_march: of its two kernels) from a committed ncu capture, if it was taken on
+    the current sources."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as fh:
             d = json.load(fh)
-        e = d.get(kernel_key)
-        if e and e.get("source_hash") == source_hash("k_step_ip" if kernel_key.startswith("k_step_ip") else "k_step"):
+        e = d.get(f"{kernel}_{key}")
+        if e and e.get("source_hash") == source_hash(kernel):
             return float(e["bytes_per_launch"])
     except Exception:
         pass
@@ -361,9 +363,9 @@ def thermal_form(lbm, L, steps, warmup, local_rank):
             stop.record(stream)
             stop.synchronize()
         lat.sync()
+        bpl *= passes_per_step(lat, steps)
         lat.close()
         ms = start.elapsed_time(stop)
-        bpl /= steps_per_pass(prec, L * L, 13, plain=False)
         bw = bpl * L * L * steps / (ms * 1e-3) / 1e9
         out[prec] = {"value": L * L * steps / (ms * 1e-3) / 1e6, "unit": "MLUPS", "achieved_gbs": bw, "roofline_frac": bw / peak,
                      "algorithmic_bytes_per_lu": bpl, "steps": steps, "clocks": clk.summary()}
@@ -401,9 +403,9 @@ def heterogeneous_form(lbm, L, steps, warmup, local_rank):
             stop.record(stream)
             stop.synchronize()
         lat.sync()
+        bpl *= passes_per_step(lat, steps) or 1.0
         lat.close()
         ms = start.elapsed_time(stop)
-        bpl /= steps_per_pass(prec, L * L, plain=False)
         bw = bpl * L * L * steps / (ms * 1e-3) / 1e9
         out[name] = {"value": L * L * steps / (ms * 1e-3) / 1e6, "unit": "MLUPS", "achieved_gbs": bw, "roofline_frac": bw / peak,
                      "algorithmic_bytes_per_lu": bpl, "steps": steps, "clocks": clk.summary()}
@@ -431,6 +433,7 @@ def ensemble_form(lbm, steps, local_rank):
         nt, k, _ = b.tune(steps=8)
         tiling = "flat" if b.get_tiling() == lbm.TILING_FLAT else "rows"
         ipc = b.get_items_per_cta()
+        per_launch = b.get_steps_per_launch()
         b.step(32)
         b.sync()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -450,12 +453,12 @@ def ensemble_form(lbm, steps, local_rank):
         b.sync()
         b.close()
         bpl = BYTES_PER_LU[prec] + 8  # + per-cell eps and K
-        if key == "fp32":
-            bpl /= steps_per_pass(prec, cells, plain=False)
+        bpl /= per_launch
         mlups = cells * steps / (ms_b * 1e-3) / 1e6
         res[key] = {"batched_MLUPS": mlups, "one_by_one_MLUPS": cells * each / (ms_e * 1e-3) / 1e6,
                     "batched_roofline_frac": mlups * 1e6 * bpl / 1e9 / peak, "algorithmic_bytes_per_lu": bpl,
-                    "launch": {"threads_per_cta": nt, "ctas_per_sm": k, "items_per_cta": ipc, "tiling": tiling},
+                    "launch": {"steps_per_launch": per_launch,
+                               **({} if per_launch > 1 else {"threads_per_cta": nt, "ctas_per_sm": k, "items_per_cta": ipc, "tiling": tiling})},
                     "steps": steps,
                     "one_by_one_steps": each,
                     "device_bytes": device_bytes, "clocks": clk.summary()}
@@ -528,6 +531,8 @@ def run_gpu(args, rank, world, local_rank):
         ms = max_over_ranks(ms, dist, "cuda")
         dist.barrier()
     cells = L * L
+    steps_per_launch, launches = lat.step_plan(args.steps)
+    passes = passes_per_step(lat, args.steps)
     mlups = cells * args.steps * world / (ms * 1e-3) / 1e6
 
     # end to end through the C-ABI with host buffers: each step takes its wall velocities from
@@ -604,19 +609,18 @@ def run_gpu(args, rank, world, local_rank):
             if other == prec:
                 continue
             ms_o, clk_o, lat_o = timed_steps(lbm, L, other, max(3, args.steps // 2), args.warmup, local_rank, dist)
+            bpl_o = BYTES_PER_LU[other] * (passes_per_step(lat_o, max(3, args.steps // 2)) or 1.0)
             lat_o.close()
-            bpl_o = BYTES_PER_LU[other] / (1 if streaming else steps_per_pass(other, cells, sides=args.walls))
             bw = bpl_o * cells / (ms_o * 1e-3 / max(3, args.steps // 2)) / 1e9
             forms[other] = {"value": cells * max(3, args.steps // 2) / (ms_o * 1e-3) / 1e6, "unit": "MLUPS",
                             "roofline_frac": bw / peak, "achieved_gbs": bw, "algorithmic_bytes_per_lu": bpl_o,
                             "clocks": clk_o}
     if rank != 0:
         return 0
-    per_pass = 1 if streaming else steps_per_pass(prec, cells, sides=args.walls)
-    bpl = BYTES_PER_LU[prec] / per_pass
-    achieved = bpl * cells / (ms * 1e-3 / args.steps) / 1e9
-    kernel_key = (f"k_step_{prec}_uniform_{L}" if not streaming else f"k_step_ip_{prec}_uniform_{L}") + ("_nee" if args.walls == "nee" else "")
-    traffic = traffic_for(kernel_key)
+    kernel = "k_step_ip" if streaming else {1: "k_step", 2: "k_march"}.get(steps_per_launch, "k_tile")
+    bpl = BYTES_PER_LU[prec] * (passes or 1.0)
+    achieved = bpl * cells / (ms * 1e-3 / args.steps) / 1e9 if passes else None  # (a tile's state stays in L2)
+    traffic = traffic_for(kernel, f"{prec}_uniform_{L}" + ("_nee" if args.walls == "nee" else ""))
     line = {
         "metric": METRIC, "value": mlups, "unit": "MLUPS", "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -627,10 +631,10 @@ def run_gpu(args, rank, world, local_rank):
                    "nx": L, "ny": L, "precision": prec,
                    "l2": f"inputs larger than L2 ({1 if streaming else 2} population buffer(s) of {BYTES_PER_LU[prec] // 2 * cells / 1e6:.0f} MB)",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": traffic, "peak_source": f"{peak_kind} hbm_gbs", "kernel": "k_step_ip" if streaming else "k_march" if per_pass == 2 else "k_step",
+        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak if passes else None,
+                     "traffic": traffic, "peak_source": f"{peak_kind} hbm_gbs", "kernel": kernel,
                      "algorithmic_bytes_per_lu": bpl},
-        "gpu_launches": args.steps,
+        "gpu_launches": launches,
         "e2e": {"value": e2e_mlups, "unit": "MLUPS", "h2d_bytes_per_step": int(walls.numel() * 4),
                 "d2h_bytes_per_step": int(probe.numel() * 4), "steps": e2e_steps,
                 "call": "lbm_set_walls(pinned host) + lbm_step(1) + lbm_probe_async(pinned host) per step; the host reads "
@@ -671,13 +675,15 @@ def run_case(args, local_rank):
         L, _, _ = lat.adjoint(64, "flux")
         lat.close()
         print(json.dumps({"case": "adjoint", "loss": L}))
-    elif args.case == "batch":  # 64 lattices of the ensemble (--precision), one 64-thread CTA per work item
+    elif args.case in ("batch", "batch_pairs"):  # 64 lattices of the ensemble (--precision), one 64-thread CTA per
+                                                 # work item, or (FP32) two steps per launch
         cfgs, media = workloads.ensemble(lbm, n=64, seed=42, precision=PREC[args.precision])
         b = workloads.build(lbm, cfgs, media)
-        b.set_launch(64, 0)
+        if args.case == "batch":
+            b.set_launch(64, 0)
         b.step(8)
         b.sync()
-        print(json.dumps({"case": "batch", **b.info()}))
+        print(json.dumps({"case": args.case, "steps_per_launch": b.get_steps_per_launch(), **b.info()}))
         b.close()
     elif args.case == "nusselt":  # natural convection run to steady state, Nu vs Table 1 (3.451)
         L = args.size
@@ -729,14 +735,14 @@ def run_sweep(args, local_rank):
             steps = min(steps, 64000) // 32 * 32
             ms, clk, lat = timed_steps(lbm, L, prec, steps, args.warmup, local_rank,
                                        streaming=1 if args.streaming == "inplace" else 0, walls=args.walls)
+            passes = passes_per_step(lat, steps)
             lat.close()
             cells = L * L
-            per_pass = 1 if args.streaming == "inplace" else steps_per_pass(prec, cells, sides=args.walls)
-            bw = BYTES_PER_LU[prec] / per_pass * cells * steps / (ms * 1e-3) / 1e9
+            bw = BYTES_PER_LU[prec] * passes * cells * steps / (ms * 1e-3) / 1e9 if passes else None
             l2 = 2 * BYTES_PER_LU[prec] // 2 * cells / 1e6
             print(json.dumps({"size": L, "precision": prec, "streaming": args.streaming, "steps": steps,
                               "MLUPS": cells * steps / (ms * 1e-3) / 1e6,
-                              "achieved_gbs": bw, "roofline_frac": bw / peak, "peak_source": peak_kind,
+                              "achieved_gbs": bw, "roofline_frac": bw / peak if passes else None, "peak_source": peak_kind,
                               "state_MB": l2, "l2_resident": l2 < 129.0, "clocks": clk}), flush=True)
             torch.cuda.empty_cache()
     return 0
@@ -760,7 +766,7 @@ def main():
     ap.add_argument("--adjoint-steps", type=int, default=4000, help="T of the adjoint form")
     ap.add_argument("--ensemble-steps", type=int, default=10000, help="steps of the 512-lattice ensemble form")
     ap.add_argument("--adjoint-nx", type=int, default=1024, help="channel length of --case adjoint (height nx / 2)")
-    ap.add_argument("--case", default="", choices=["", "adjoint", "batch", "fp16", "thermal", "nusselt", "inplace"],
+    ap.add_argument("--case", default="", choices=["", "adjoint", "batch", "batch_pairs", "fp16", "thermal", "nusselt", "inplace"],
                     help="run one small case of a kernel family (for profiler captures) and exit")
     ap.add_argument("--sweep", default="", help="comma-separated lattice sizes: print one line per size and precision")
     args = ap.parse_args()

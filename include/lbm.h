@@ -169,6 +169,10 @@ LBM_API int lbm_init_temperature(lbm_ctx* ctx, double T_init);
  * (so a context on the legacy default stream works too); lbm_set_medium discards the captured graphs. */
 LBM_API int lbm_step(lbm_ctx* ctx, int n);
 
+/* How lbm_step(ctx, n) would run now: the most steps that one launch takes (1, 2 or 4, see lbm_step)
+ * and the kernels that the call launches.  Either output may be NULL; nothing is launched. */
+LBM_API int lbm_step_plan(const lbm_ctx* ctx, int n, int* steps_per_launch, int64_t* launches);
+
 /* Replace the wall velocities u_wall[4][2] (left, right, bottom, top; float32, host or device)
  * for the following steps -- e.g. a time-dependent lid.  The copy is enqueued on the stream. */
 LBM_API int lbm_set_walls(lbm_ctx* ctx, const float* u_wall);

@@ -757,6 +757,29 @@ int lbm_step(lbm_ctx* c, int n) {
   return LBM_OK;
 }
 
+int lbm_step_plan(const lbm_ctx* c, int n, int* steps_per_launch, int64_t* launches) {
+  if (!c) return fail(LBM_EINVAL, "null context");
+  if (n < 0) return fail(LBM_EINVAL, "negative step count");
+  const Pace pace = pace_of(c);
+  if (steps_per_launch) *steps_per_launch = pace.most;
+  if (!launches) return LBM_OK;
+  const int one = c->inplace && c->edge ? 2 : 1;
+  if (pace.most == 1) {
+    *launches = (int64_t)n * one;
+    return LBM_OK;
+  }
+  // (run_steps: whole launches, the rest of the first n - 1 steps, the last step)
+  const int several = pace.tile ? 1 : march_kernels(params_for(c), c->prec, c->het, thermal_of(c));
+  const int graphs = n > pace.graph ? (n - 1) / pace.graph : 0, left = n - graphs * pace.graph;
+  *launches = (int64_t)graphs * (pace.graph / pace.most) * several;
+  if (left > 1) {
+    const int k = (left - 1) / pace.most, rest = (left - 1) % pace.most;
+    *launches += (int64_t)k * several + (rest > 1 ? several : rest);
+  }
+  if (left > 0) *launches += one;
+  return LBM_OK;
+}
+
 int lbm_set_walls(lbm_ctx* c, const float* u_wall) {
   if (!c || !u_wall) return fail(LBM_EINVAL, "null argument");
   const int kind = pointer_kind(c, u_wall);

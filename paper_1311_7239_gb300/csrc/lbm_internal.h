@@ -62,6 +62,7 @@ int sm_count();  // SMs of the current device
 constexpr uint64_t kMarchBytes = 100ull << 20;  // FP32 state (both buffers) from which steps are taken in pairs
 bool march_shape(const StepParams& P, int prec, bool het, bool thermal);
 bool march_takes(const StepParams& P, int prec, bool het, bool thermal);
+int march_kernels(const StepParams& P, int prec, bool het, bool thermal);
 // A warp's work in the batched pair kernels: rows [ya, yb) (none if equal) of a strip of a lattice.
 struct MarchItem {
   int lattice, strip, ya, yb, strips, wrap;

@@ -427,8 +427,9 @@ int sm_count() {
   return n;
 }
 
-template <int PREC, bool HET, bool THERMAL, int C, int STAGES, int CTAS>
-static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
+// Strips and segments for CTAS resident CTAs per SM.
+template <int PREC, int C, int CTAS>
+static March march_of(const StepParams& P) {
   March M;
   M.wrap = P.bc_x == BC_PERIODIC;
   M.strips = march_strips<PREC, C>(P.nx, M.wrap);
@@ -450,6 +451,12 @@ static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
   M.side_rows = 8;
   M.segs = (ny + M.rows - 1) / M.rows;
   M.side_segs = (ny + M.side_rows - 1) / M.side_rows;
+  return M;
+}
+
+template <int PREC, bool HET, bool THERMAL, int C, int STAGES, int CTAS>
+static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
+  const March M = march_of<PREC, C, CTAS>(P);
   const size_t bytes = (kMarchThreads / 32) * STAGES * Marcher<PREC, HET, THERMAL, C, STAGES, false, false>::kStage;
   auto side = k_march_side<PREC, HET, THERMAL, C, STAGES, false>;
   if constexpr (PREC == PREC_FP32 && !THERMAL) {
@@ -467,16 +474,23 @@ static cudaError_t launch_march_t(const StepParams& P, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// cells per lane and CTAs per SM: the widest forms that hold their registers without a spill (any
+// spill costs more than a missing CTA: local memory shares the little L1 that the stages leave)
 template <int PREC>
 static cudaError_t launch_march_p(const StepParams& P, bool het, bool thermal, cudaStream_t s) {
-  // cells per lane and CTAs per SM: the widest forms that hold their registers without a spill (any
-  // spill costs more than a missing CTA: local memory shares the little L1 that the stages leave)
   if constexpr (PREC == PREC_FP32) {
     if (thermal) return launch_march_t<PREC, false, true, 2, 3, 4>(P, s);
     return het ? launch_march_t<PREC, true, false, 2, 3, 4>(P, s) : launch_march_t<PREC, false, false, 4, 3, 3>(P, s);
   } else {
     return launch_march_t<PREC, false, false, 4, 3, 3>(P, s);
   }
+}
+
+// kernels of launch_march: the sides', and the main one where the lattice has strips without a side
+int march_kernels(const StepParams& P, int prec, bool het, bool thermal) {
+  const March M = prec == PREC_FP32 ? (het || thermal ? march_of<PREC_FP32, 2, 4>(P) : march_of<PREC_FP32, 4, 3>(P))
+                                    : march_of<PREC_FP16, 4, 3>(P);
+  return M.s1 > M.s0 ? 2 : 1;
 }
 
 cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, cudaStream_t s) {

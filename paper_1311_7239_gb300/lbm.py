@@ -81,6 +81,7 @@ SIGNATURES = {
     "lbm_init_equilibrium": (ctypes.c_int, [_c_ctx, ctypes.c_double, ctypes.c_double, ctypes.c_double, ctypes.c_int]),
     "lbm_init_temperature": (ctypes.c_int, [_c_ctx, ctypes.c_double]),
     "lbm_step": (ctypes.c_int, [_c_ctx, ctypes.c_int]),
+    "lbm_step_plan": (ctypes.c_int, [_c_ctx, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int64)]),
     "lbm_set_walls": (ctypes.c_int, [_c_ctx, _f32p]),
     "lbm_probe": (ctypes.c_int, [_c_ctx, ctypes.c_int, ctypes.c_int, _f32p]),
     "lbm_probe_async": (ctypes.c_int, [_c_ctx, ctypes.c_int, ctypes.c_int, _f32p]),
@@ -257,6 +258,12 @@ class Lattice:
     # time stepping --------------------------------------------------------------------------
     def step(self, n=1):
         _check(lib().lbm_step(self._h, int(n)), "lbm_step")
+
+    def step_plan(self, n=1):
+        """(the most steps that a launch of ``step(n)`` takes, the kernels that it launches)."""
+        k, m = ctypes.c_int(), ctypes.c_int64()
+        _check(lib().lbm_step_plan(self._h, int(n), ctypes.byref(k), ctypes.byref(m)), "lbm_step_plan")
+        return k.value, m.value
 
     def sync(self):
         _check(lib().lbm_sync(self._h), "lbm_sync")
