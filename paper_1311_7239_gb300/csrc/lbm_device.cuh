@@ -502,8 +502,8 @@ __device__ __forceinline__ void collide_pair(float2 d[8], const PairCoef& c, flo
 }
 
 // collide_d2q8 for two cells at once on the packed FP32 pairs, in true units and with the roundings
-// of the scalar form operation by operation (the multiply-adds it is compiled to, written out), so
-// that both give the same bits: FP32 storage may take either.  Differences are multiply-adds by -1,
+// of the scalar form operation by operation, so that both give the same bits: FP32 storage may take
+// either.  Differences are multiply-adds by -1,
 // since the packed instructions have no negated operands.
 struct PairMedium {
   float2 phi, inv_phi, l0, l1, nclin, ncnl, s_v;  // l0 = 1/2 + c_lin / 4, l1 = c_nl / 2, -c_lin, -c_nl

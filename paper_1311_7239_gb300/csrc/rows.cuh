@@ -291,62 +291,62 @@ struct RowOps {
       }
     }
 #pragma unroll
-      for (int h = 0; h < C / 2; ++h) {
-        const int ca = 2 * h, cb = ca + 1;
-        float da[8], db[8], ga[5], gb[5];
+    for (int h = 0; h < C / 2; ++h) {
+      const int ca = 2 * h, cb = ca + 1;
+      float da[8], db[8], ga[5], gb[5];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          da[i] = get_cell<PREC, C>(w[i], ca, P.inv_scale);
-          db[i] = get_cell<PREC, C>(w[i], cb, P.inv_scale);
-        }
-        if constexpr (THERMAL) {
+      for (int i = 0; i < 8; ++i) {
+        da[i] = get_cell<PREC, C>(w[i], ca, P.inv_scale);
+        db[i] = get_cell<PREC, C>(w[i], cb, P.inv_scale);
+      }
+      if constexpr (THERMAL) {
 #pragma unroll
-          for (int i = 0; i < 5; ++i) {
-            ga[i] = get_cell<PREC, C>(gw[i], ca, P.inv_scale);
-            gb[i] = get_cell<PREC, C>(gw[i], cb, P.inv_scale);
-          }
-        }
-        patch_cell(ca, y, e, eg, da, ga);
-        patch_cell(cb, y, e, eg, db, gb);
-        Coef ma, mb;
-        if constexpr (HET) {
-          const float* sv = P.sv ? P.sv + (int64_t)in_rows(y) * P.pitch : nullptr;
-          ma = coef_of(P, ph[ca], k[ca], sv ? __ldg(sv + in_cols(col(ca), 1)) : P.s_v);
-          mb = coef_of(P, ph[cb], k[cb], sv ? __ldg(sv + in_cols(col(cb), 1)) : P.s_v);
-        } else {
-          ma = mb = coef_uniform(P);
-        }
-        if constexpr (kPressure) {
-          if (inlet && h == 0) pressure_cell(P, db, mb, ma, P.p_in, da);
-          if (outlet && cr == ca) pressure_cell(P, inner, HET ? coef_of(P, inner_ph, inner_k, P.s_v) : ma, ma, P.p_out, da);
-          if (outlet && cr == cb) pressure_cell(P, da, ma, mb, P.p_out, db);
-        }
-        const PairMedium m = pair_medium(ma, mb);
-        float2 d[8], g[5], n0, ay = f2(P.ay), ux, uy;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) d[i] = make_float2(da[i], db[i]);
-        if constexpr (THERMAL) {
-#pragma unroll
-          for (int i = 0; i < 5; ++i) g[i] = make_float2(ga[i], gb[i]);
-          n0 = add2(add2(add2(add2(g[0], g[1]), g[2]), g[3]), g[4]);
-          ay = fma2(f2(P.g_beta), n0, ay);  // a = g beta (T - T0) j
-        }
-        collide_d2q8_pair(d, m, P.ax, ay, P, ux, uy);
-        check += (fabsf(ux.x) + fabsf(uy.x)) + (fabsf(ux.y) + fabsf(uy.y));
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          put_cell<PREC, C>(w[i], ca, d[i].x, P.scale);
-          put_cell<PREC, C>(w[i], cb, d[i].y, P.scale);
-        }
-        if constexpr (THERMAL) {
-          collide_d2q5_pair_fp32(g, n0, ux, uy, P);
-#pragma unroll
-          for (int i = 0; i < 5; ++i) {
-            put_cell<PREC, C>(gw[i], ca, g[i].x, P.scale);
-            put_cell<PREC, C>(gw[i], cb, g[i].y, P.scale);
-          }
+        for (int i = 0; i < 5; ++i) {
+          ga[i] = get_cell<PREC, C>(gw[i], ca, P.inv_scale);
+          gb[i] = get_cell<PREC, C>(gw[i], cb, P.inv_scale);
         }
       }
+      patch_cell(ca, y, e, eg, da, ga);
+      patch_cell(cb, y, e, eg, db, gb);
+      Coef ma, mb;
+      if constexpr (HET) {
+        const float* sv = P.sv ? P.sv + (int64_t)in_rows(y) * P.pitch : nullptr;
+        ma = coef_of(P, ph[ca], k[ca], sv ? __ldg(sv + in_cols(col(ca), 1)) : P.s_v);
+        mb = coef_of(P, ph[cb], k[cb], sv ? __ldg(sv + in_cols(col(cb), 1)) : P.s_v);
+      } else {
+        ma = mb = coef_uniform(P);
+      }
+      if constexpr (kPressure) {
+        if (inlet && h == 0) pressure_cell(P, db, mb, ma, P.p_in, da);
+        if (outlet && cr == ca) pressure_cell(P, inner, HET ? coef_of(P, inner_ph, inner_k, P.s_v) : ma, ma, P.p_out, da);
+        if (outlet && cr == cb) pressure_cell(P, da, ma, mb, P.p_out, db);
+      }
+      const PairMedium m = pair_medium(ma, mb);
+      float2 d[8], g[5], n0, ay = f2(P.ay), ux, uy;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) d[i] = make_float2(da[i], db[i]);
+      if constexpr (THERMAL) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) g[i] = make_float2(ga[i], gb[i]);
+        n0 = add2(add2(add2(add2(g[0], g[1]), g[2]), g[3]), g[4]);
+        ay = fma2(f2(P.g_beta), n0, ay);  // a = g beta (T - T0) j
+      }
+      collide_d2q8_pair(d, m, P.ax, ay, P, ux, uy);
+      check += (fabsf(ux.x) + fabsf(uy.x)) + (fabsf(ux.y) + fabsf(uy.y));
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        put_cell<PREC, C>(w[i], ca, d[i].x, P.scale);
+        put_cell<PREC, C>(w[i], cb, d[i].y, P.scale);
+      }
+      if constexpr (THERMAL) {
+        collide_d2q5_pair_fp32(g, n0, ux, uy, P);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+          put_cell<PREC, C>(gw[i], ca, g[i].x, P.scale);
+          put_cell<PREC, C>(gw[i], cb, g[i].y, P.scale);
+        }
+      }
+    }
     return check;
   }
 
