@@ -183,13 +183,14 @@ int set_launch(lbm_batch* b, int nt, int ctas_per_sm) {
 }
 
 // One batched step from buffer parity `cur` on stream s, in the form the launch shape selects.
-cudaError_t launch_batch(const lbm_batch* b, int cur, cudaStream_t s) {
+// graph: the launch is captured into one.
+cudaError_t launch_batch(const lbm_batch* b, int cur, cudaStream_t s, bool graph = false) {
   if (b->inplace)
     return launch_step_batch_inplace(b->dp[cur], b->item_start, b->item_lattice, b->total_items, b->prec, cur, s);
   const bool per_item = b->ctas_per_sm == 0 && b->items_per_cta == 1;
   if (b->shared_consts && per_item)
     return launch_step_batch_shared(b->hp[0][0], b->rec[cur], b->dp[cur], b->item_start, b->item_lattice, b->total_items, b->prec,
-                                    b->nt, b->flat, s);
+                                    b->nt, b->flat, graph, s);
   // otherwise the range walk: a persistent grid, or ceil(items / items_per_cta) CTAs
   return launch_step_batch(b->dp[cur], b->item_start, per_item ? b->item_lattice : nullptr, b->n, b->total_items, b->prec, b->nt,
                            b->grid, b->flat, s);
@@ -234,7 +235,7 @@ int capture(lbm_batch* b, int cur) {
   LBM_BCUDA(cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
   cudaError_t le = cudaSuccess;
   for (int k = 0; k < (b->pairs ? kBatchGraphSteps / 2 : kBatchGraphSteps) && le == cudaSuccess; ++k)
-    le = b->pairs ? launch_pair(b, cur ^ (k & 1), b->capture_stream) : launch_batch(b, cur ^ (k & 1), b->capture_stream);
+    le = b->pairs ? launch_pair(b, cur ^ (k & 1), b->capture_stream) : launch_batch(b, cur ^ (k & 1), b->capture_stream, true);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(b->capture_stream, &g);
   if (le != cudaSuccess || e != cudaSuccess) {

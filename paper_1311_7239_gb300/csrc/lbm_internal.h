@@ -53,7 +53,7 @@ struct BatchRec {
 
 int64_t batch_items(int nx, int ny, int bc_y, int nt, int flat);
 cudaError_t launch_step_batch_shared(const StepParams& U, const BatchRec* R, const StepParams* Pd, const int64_t* item_start,
-                                     const int* item_lattice, int64_t total, int prec, int nt, int flat, cudaStream_t s);
+                                     const int* item_lattice, int64_t total, int prec, int nt, int flat, bool graph, cudaStream_t s);
 int batch_max_ctas_per_sm(int prec, int nt);
 cudaError_t launch_step_batch(const StepParams* Pd, const int64_t* item_start, const int* item_lattice, int n, int64_t total, int prec,
                               int nt, int grid, int flat, cudaStream_t s);

@@ -361,13 +361,13 @@ __global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 896 : 768) / NT) k_st
 // parameters, by value: the kernel's constant bank) supplies those and the collision constants, the
 // record of the item's lattice the fields that differ, so a main item starts its gathers without
 // staging the parameter set in shared memory and keeps the constants out of the registers.  Frame
-// items, which use every parameter, stage the lattice's set as the general form.  Register caps:
-// FP16 and BF16 at 72 registers (FP16, 512 lattices: 122.1 GLUPS, 117.7 at 64, 112.9 at 80, the staged
-// form 102.4; BF16, 128 lattices of 64..512 cells a side: 109.3 us per step, 114.2 at 64, 118.1 at 80),
-// FP32 at 64 (the same 128 lattices 138.4, 138.5 at 72; 8 lattices of 64..256, whose CTAs just fit the
-// chip at once, 5.9, 7.0 at 72).
+// items, which use every parameter, stage the lattice's set as the general form.  Held to 72 registers
+// (FP16, 512 lattices: 122.1 GLUPS, 117.7 at 64, 112.9 at 80, the staged form 102.4; 128 lattices of
+// 64..512 cells a side: BF16 109.3 us per step, 114.2 at 64, 118.1 at 80, FP32 138.9, 144.7 at 64).
+constexpr int kSharedThreads = 896;  // threads per SM at 72 registers
+
 template <int PREC, int NT>
-__global__ void __launch_bounds__(NT, (PREC == PREC_FP32 ? 1024 : 896) / NT)
+__global__ void __launch_bounds__(NT, kSharedThreads / NT)
     k_step_batch_items_shared(const StepParams U, const BatchRec* __restrict__ R, const StepParams* __restrict__ Pd,
                               const int64_t* __restrict__ item_start, const int* __restrict__ item_lattice, int flat) {
   launch_dependents();
@@ -470,21 +470,36 @@ static cudaError_t launch_batch_p(const StepParams* Pd, const int64_t* item_star
   return cudaGetLastError();
 }
 
+template <int PREC, int NT>
+static cudaError_t launch_shared_t(const StepParams& U, const BatchRec* R, const StepParams* Pd, const int64_t* item_start,
+                                   const int* item_lattice, int64_t total, int flat, bool graph, cudaStream_t s) {
+  const auto fn = k_step_batch_items_shared<PREC, NT>;
+  // Launched early, but not within a graph where the chip holds one step's CTAs at once and not two
+  // steps': the next step's would then crowd on the SMs that have room (FP32 lattices of 64..256 cells a
+  // side, eight: 7.3 -> 6.5 us per step, twelve: 7.25 -> 6.85, sixteen, which all but fill the chip: 7.34,
+  // 7.42 so; eight by single launches 7.7, against 8.3 one after the other).
+  const int64_t room = (int64_t)sm_count() * (kSharedThreads / NT);
+  if (!graph || 2 * total <= room || 8 * total >= 7 * room)
+    return launch_early(fn, dim3((unsigned)total), dim3(NT), 0, s, U, R, Pd, item_start, item_lattice, flat);
+  fn<<<(unsigned)total, NT, 0, s>>>(U, R, Pd, item_start, item_lattice, flat);
+  return cudaGetLastError();
+}
+
 template <int PREC>
 static cudaError_t launch_shared_p(const StepParams& U, const BatchRec* R, const StepParams* Pd, const int64_t* item_start,
-                            const int* item_lattice, int64_t total, int nt, int flat, cudaStream_t s) {
+                                   const int* item_lattice, int64_t total, int nt, int flat, bool graph, cudaStream_t s) {
   switch (nt) {
-    case 64: return launch_early(k_step_batch_items_shared<PREC, 64>, dim3((unsigned)total), dim3(64), 0, s, U, R, Pd, item_start, item_lattice, flat);
-    case 256: return launch_early(k_step_batch_items_shared<PREC, 256>, dim3((unsigned)total), dim3(256), 0, s, U, R, Pd, item_start, item_lattice, flat);
-    default: return launch_early(k_step_batch_items_shared<PREC, 128>, dim3((unsigned)total), dim3(128), 0, s, U, R, Pd, item_start, item_lattice, flat);
+    case 64: return launch_shared_t<PREC, 64>(U, R, Pd, item_start, item_lattice, total, flat, graph, s);
+    case 256: return launch_shared_t<PREC, 256>(U, R, Pd, item_start, item_lattice, total, flat, graph, s);
+    default: return launch_shared_t<PREC, 128>(U, R, Pd, item_start, item_lattice, total, flat, graph, s);
   }
 }
 
 cudaError_t launch_step_batch_shared(const StepParams& U, const BatchRec* R, const StepParams* Pd, const int64_t* item_start,
-                                     const int* item_lattice, int64_t total, int prec, int nt, int flat, cudaStream_t s) {
-  if (prec == PREC_FP16) return launch_shared_p<PREC_FP16>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
-  if (prec == PREC_BF16) return launch_shared_p<PREC_BF16>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
-  return launch_shared_p<PREC_FP32>(U, R, Pd, item_start, item_lattice, total, nt, flat, s);
+                                     const int* item_lattice, int64_t total, int prec, int nt, int flat, bool graph, cudaStream_t s) {
+  if (prec == PREC_FP16) return launch_shared_p<PREC_FP16>(U, R, Pd, item_start, item_lattice, total, nt, flat, graph, s);
+  if (prec == PREC_BF16) return launch_shared_p<PREC_BF16>(U, R, Pd, item_start, item_lattice, total, nt, flat, graph, s);
+  return launch_shared_p<PREC_FP32>(U, R, Pd, item_start, item_lattice, total, nt, flat, graph, s);
 }
 
 // Largest number of CTAs of the persistent batched kernel (prec, nt) resident on one SM.
