@@ -12,10 +12,10 @@
 // 4096^2 FP32, interior alone, 183 GLUPS against 161 with the rows prefetched in registers.
 // The collisions run on packed FP32 pairs (collide_d2q8_pair, collide_pair): with scalar ones the
 // pass was bound by instruction issue (79 %, 195 thread instructions per cell and step).
-// Measured (GLUPS, one step per pass -> two): FP32 4096^2 104 -> 177, per-cell medium 91 -> 148,
-// temperature (2048^2) 59 -> 90, FP16 4096^2 176 -> 208.  What bounds it now: HBM at 32 bytes per cell and
-// step (83 % of the measured copy rate), with 16-bit storage the FP32 pipe and its latency (63 % busy, 12
-// warps per SM).  Every cell is rounded as by k_step: the results are the same bits.
+// Measured (GLUPS, one step per pass -> two): FP32 4096^2 104 -> 183, per-cell medium 91 -> 151,
+// temperature (2048^2) 59 -> 89, FP16 4096^2 176 -> 207.  What bounds it now: HBM at 32 bytes per cell and
+// step (86 % of the measured copy rate), with 16-bit storage latency and issue (2048^2: an instruction in
+// 56 % of the active cycles from 9 warps per SM, DRAM at a quarter of its rate).  Every cell is rounded as by k_step: the results are the same bits.
 #include "lbm_internal.h"
 #include "rows.cuh"
 
@@ -503,8 +503,9 @@ cudaError_t launch_march(const StepParams& P, int prec, bool het, bool thermal, 
 
 // --------------------------------------------------------------------------------------------
 // Batched ensembles (FP32, per-cell media): the same pairs of steps for all lattices of a batch in one
-// launch of each kernel (48 lattices of 64..1024 cells a side: 84 -> 104 GLUPS; segments of 24 rows, 8
-// at the sides: 32 and 16 rows gave 106, but 72 against 76 on lattices up to 512).  A CTA's four warps take four items of one lattice, whose parameters are
+// launch of each kernel (48 lattices of 64..1024 cells a side: 84 -> 104 GLUPS, 109 since the side warps of
+// batches without pressure columns leave their rules out; segments of 24 rows, 8 at the sides: 32 and 16
+// rows gave 106 against the 104, but 72 against 76 on lattices up to 512).  A CTA's four warps take four items of one lattice, whose parameters are
 // staged in shared memory; the items of a lattice are padded to whole CTAs.
 // --------------------------------------------------------------------------------------------
 constexpr int kBatchC = 2, kBatchStages = 3;
