@@ -239,7 +239,8 @@ LBM_API int lbm_residual_noalloc(const float* ux, const float* uy, const float* 
  * states of one segment are recomputed, on a second stream of lower priority, while the adjoint
  * steps of the next run on a stream of higher priority), two FP32 adjoint states and the gradient
  * sums (FP32 partial sums over at most 64 steps, folded into FP64 totals) form a workspace that
- * stays allocated after the call, so that repeated calls (an optimisation loop) allocate nothing;
+ * stays allocated after the call, so that repeated calls (an optimisation loop) allocate nothing (a
+ * call whose T needs less uses it too, unless it is more than twice what the call needs);
  * it is counted by lbm_memory_bytes and freed by lbm_release_workspace or lbm_destroy.  The
  * forward work is about 2 T steps.
  *   target_ux, target_uy: float32 [ny][nx] (misfit loss only; host or device).
